@@ -20,7 +20,7 @@
 //
 // Partitioned inverse: the first k columns of the inverse of the unit lower
 // trapezoid [[L11, 0], [L21, I]], X_t = [L11^{-1}; -L21 L11^{-1}] (f x k,
-// column-major), and 1/D are written to the factor arrays (FP64 or FP32),
+// grouped layout of kernels.cuh), and 1/D are written to the factor arrays (FP64 or FP32),
 // with X_t^T beside X_t for the backward sweep.
 #include <cuda_runtime.h>
 
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(FA_THREADS) k_fa_schur(const int4* __restrict_
 template <typename T, typename V>
 __global__ void k_fa_inverse(const int* __restrict__ list, const int* __restrict__ kk, const int* __restrict__ ff,
                              const int64_t* __restrict__ Foff, const int64_t* __restrict__ Moff,
-                             const int64_t* __restrict__ Doff, T* __restrict__ F, V* __restrict__ M,
+                             const int64_t* __restrict__ MToff, const int64_t* __restrict__ Doff, T* __restrict__ F, V* __restrict__ M,
                              V* __restrict__ MT, V* __restrict__ Dinv) {
   extern __shared__ __align__(16) unsigned char fa_smem[];
   T* col = reinterpret_cast<T*>(fa_smem);
@@ -339,13 +339,12 @@ __global__ void k_fa_inverse(const int* __restrict__ list, const int* __restrict
     __syncthreads();
   }
   V* Mt = M + Moff[t];
-  V* MTt = MT + Moff[t];
+  V* MTt = MT + MToff[t];
   const int64_t fk = (int64_t)f * k;
   for (int64_t i = threadIdx.x; i < fk; i += blockDim.x) {
     const int r = (int)(i % f), c = (int)(i / f);
     const double2 v = r == c ? make_double2(1.0, 0.0) : (r < c ? make_double2(0.0, 0.0) : to_d(Ft[i]));
-    Mt[i] = from_d2<V>(v);
-    MTt[c + (int64_t)r * k] = from_d2<V>(v);
+    mf_store(Mt, MTt, f, k, r, c, from_d2<V>(v));
   }
 }
 
@@ -484,7 +483,7 @@ __global__ void __launch_bounds__(FA_THREADS) k_fa_inv_update(const int4* __rest
 template <typename T, typename V>
 __global__ void k_fa_store(const int* __restrict__ list, const int* __restrict__ kk, const int* __restrict__ ff,
                            const int64_t* __restrict__ Foff, const int64_t* __restrict__ Moff,
-                           const int64_t* __restrict__ Doff, const T* __restrict__ F, V* __restrict__ M,
+                           const int64_t* __restrict__ MToff, const int64_t* __restrict__ Doff, const T* __restrict__ F, V* __restrict__ M,
                            V* __restrict__ MT, V* __restrict__ Dinv) {
   const int t = list[blockIdx.x];
   const int f = ff[t], k = kk[t];
@@ -492,13 +491,12 @@ __global__ void k_fa_store(const int* __restrict__ list, const int* __restrict__
   for (int j = threadIdx.x; j < k; j += blockDim.x)
     Dinv[Doff[t] + j] = from_d2<V>(to_d(cinv(Ft[j + (int64_t)j * f])));
   V* Mt = M + Moff[t];
-  V* MTt = MT + Moff[t];
+  V* MTt = MT + MToff[t];
   const int64_t fk = (int64_t)f * k;
   for (int64_t i = threadIdx.x; i < fk; i += blockDim.x) {
     const int r = (int)(i % f), c = (int)(i / f);
     const double2 v = r == c ? make_double2(1.0, 0.0) : (r < c ? make_double2(0.0, 0.0) : to_d(Ft[i]));
-    Mt[i] = from_d2<V>(v);
-    MTt[c + (int64_t)r * k] = from_d2<V>(v);
+    mf_store(Mt, MTt, f, k, r, c, from_d2<V>(v));
   }
 }
 
@@ -546,7 +544,7 @@ static void factor_t(DevMF& mf, double tau_abs, cudaStream_t st) {
   for (int l = 0; l < mf.nlevels; ++l) {
     const int sb = mf.fa_small_ptr_h[l], se = mf.fa_small_ptr_h[l + 1];
     if (se > sb)
-      { k_fa_inverse<T, V><<<se - sb, 256, shm, st>>>(mf.fa_small + sb, mf.k, mf.f, mf.Foff, mf.Moff, mf.Doff, F,
+      { k_fa_inverse<T, V><<<se - sb, 256, shm, st>>>(mf.fa_small + sb, mf.k, mf.f, mf.Foff, mf.Moff, mf.MToff, mf.Doff, F,
                                                       (V*)mf.M, (V*)mf.MT, (V*)mf.Dinv); count_launch(); }
     const int bb = mf.fa_big_ptr_h[l], be = mf.fa_big_ptr_h[l + 1];
     if (be == bb) continue;
@@ -559,7 +557,7 @@ static void factor_t(DevMF& mf, double tau_abs, cudaStream_t st) {
         { k_fa_inv_update<T><<<te - tb, FA_THREADS, schur_shm, st>>>(mf.fi_tiles + tb, mf.k, mf.f, mf.Foff, F,
                                                                      mf.fa_pan_off + bb, pan, l0); count_launch(); }
     }
-    { k_fa_store<T, V><<<be - bb, 256, 0, st>>>(mf.fa_big + bb, mf.k, mf.f, mf.Foff, mf.Moff, mf.Doff, F, (V*)mf.M,
+    { k_fa_store<T, V><<<be - bb, 256, 0, st>>>(mf.fa_big + bb, mf.k, mf.f, mf.Foff, mf.Moff, mf.MToff, mf.Doff, F, (V*)mf.M,
                                                 (V*)mf.MT, (V*)mf.Dinv); count_launch(); }
   }
   cudaEventRecord(ev[2], st);

@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <deque>
@@ -90,22 +91,64 @@ struct DevPool {
 };
 
 struct MFHost {
-  int64_t factor_entries = 0, front_entries = 0, stored_entries = 0;
+  int64_t factor_entries = 0, front_entries = 0;
   std::vector<int> fa_small_ptr, fa_big_ptr, fa_step_ptr, fa_tile_ptr, fi_tile_ptr;  // factorisation schedule
   int max_front = 0, nfronts = 0, nlevels = 0;
-  std::vector<int> level_ptr, ftile_ptr, btile_ptr, frb_ptr, brb_ptr;
-  std::vector<int> fs_ptr, bs_ptr, ftc_ptr, btc_ptr;  // tensor-core mode split of the tile lists
-  std::vector<int64_t> level_row;
-  // per-level algorithmic work of one solve sweep (complex multiply-adds per column)
-  std::vector<double> fwd_cmacs, bwd_cmacs;
-  // per level: every tile has at most 64 output rows (half-height tiles in the solve)
+  std::vector<int> level_ptr;
+  std::vector<int> ftask_ptr, btask_ptr, fbrows, bbrows, fgroups, bgroups;  // sweep tasks (DevMF)
+  // tensor-core form: tiles and split row blocks per level, levels whose tiles all have at most 64 rows
+  std::vector<int> frb_ptr, brb_ptr, fs_ptr, bs_ptr, ftc_ptr, btc_ptr;
   std::vector<char> fhalf, bhalf;
 };
 
 // Pack the fronts of several local matrices into one device structure;
 // sub_off[i] is the first row of subdomain i in the flat sub-vector.
-constexpr int MF_TILE_ROWS = 128;  // output rows per sweep tile (MF_TILE in mf.cu)
-constexpr int MF_TILE_K = 128;     // reduction length per sweep tile (MF_TK in mf.cu)
+constexpr int MF_TILE_ROWS = 128;  // output rows per tile of the tensor-core form (MF_TILE in mf.cu)
+constexpr int MF_TILE_K = 128;     // reduction length per tile (MF_TK in mf.cu)
+
+// Sweep tasks of one level (sweep.cu). A task is a run of 16-row groups of
+// one front. Where some reduction of the level is longer than what a CTA keeps
+// in shared memory, a task has at most four groups (one per warp, which
+// follows the input rows as they stream by), elsewhere up to 16, which share
+// one staging of the input, fewer on levels that would have less than 8 tasks
+// per SM (FP64: 16) otherwise. FP32 keeps four, one for each warp; FP64 goes
+// down to one, whose reduction the warps share. The largest fronts come first.
+void level_tasks(bool fwd, bool fp32, const int* list, int count, const std::vector<int>& k, const std::vector<int>& f,
+                 const std::vector<int64_t>& rowoff, const std::vector<int64_t>& moff,
+                 const std::vector<int64_t>& doff, std::vector<SweepTask>& tasks, int& brows, int& ngroups) {
+  int64_t groups = 0;
+  std::vector<int> order;
+  for (int q = 0; q < count; ++q) {
+    const int g = list[q], nout = fwd ? f[g] : k[g];
+    if (nout == 0) continue;
+    groups += (nout + MF_GR - 1) / MF_GR;
+    order.push_back(g);
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return (int64_t)f[a] * k[a] > (int64_t)f[b] * k[b]; });
+  brows = 0;
+  for (int g : order) brows = std::max(brows, fwd ? k[g] : f[g]);
+  const int64_t fill = groups / (fp32 ? 1216 : 2432);
+  const int most = (int)std::min<int64_t>(std::max<int64_t>(fill, fp32 ? 4 : 1), brows > MF_RES ? 4 : 16);
+  for (int g : order) {
+    const int nout = fwd ? f[g] : k[g];
+    const int ng = (nout + MF_GR - 1) / MF_GR;
+    const int nt = (ng + most - 1) / most;
+    for (int t = 0, g0 = 0; t < nt; ++t) {
+      SweepTask T;
+      T.m = moff[g];
+      T.row = rowoff[g];
+      T.d = (int32_t)doff[g];
+      T.front = g;
+      T.k = (uint16_t)k[g];
+      T.f = (uint16_t)f[g];
+      T.g0 = (uint16_t)g0;
+      T.ng = (uint16_t)((int64_t)ng * (t + 1) / nt - g0);
+      g0 += T.ng;
+      tasks.push_back(T);
+    }
+  }
+  ngroups = (int)groups;
+}
 
 void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const FrontTree*>& trees,
               const std::vector<int64_t>& sub_off, bool fp32, bool fr32, bool tc, bool persistent, DevMF& mf,
@@ -116,7 +159,7 @@ void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const Fron
   for (size_t i = 0; i < ns; ++i) base[i + 1] = base[i] + (int)trees[i]->k.size();
   const int nf = base[ns];
   std::vector<int> k(nf), f(nf), height(nf), child_ptr(nf + 1, 0), child_idx, parent(nf, -1);
-  std::vector<int64_t> Foff(nf + 1, 0), rowoff(nf + 1, 0), Moff(nf + 1, 0), Doff(nf + 1, 0);
+  std::vector<int64_t> Foff(nf + 1, 0), rowoff(nf + 1, 0), Moff(nf + 1, 0), MToff(nf + 1, 0), Doff(nf + 1, 0);
   for (size_t i = 0; i < ns; ++i) {
     const FrontTree& T = *trees[i];
     for (size_t t = 0; t < T.k.size(); ++t) {
@@ -152,13 +195,14 @@ void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const Fron
   }
   for (int g = 0; g < nf; ++g) {
     Foff[g + 1] = Foff[g] + (int64_t)f[g] * f[g];
-    Moff[g + 1] = Moff[g] + (int64_t)f[g] * k[g];
+    Moff[g + 1] = Moff[g] + mf_fwd_size(f[g], k[g]);
+    MToff[g + 1] = MToff[g] + mf_bwd_size(f[g], k[g]);
     Doff[g + 1] = Doff[g] + k[g];
     info.max_front = std::max(info.max_front, f[g]);
     if ((int64_t)f[g] * f[g] >= (int64_t)1 << 31) throw HzError{HZ_EINVAL, "front too large"};
   }
   info.front_entries = Foff[nf];
-  info.stored_entries = Moff[nf];
+  if (Doff[nf] >= (int64_t)1 << 31) throw HzError{HZ_EINVAL, "local matrices too large"};
   std::vector<int> rows(rowoff[nf]), cmap(rowoff[nf], -1);
   std::vector<int64_t> amap_ptr(nf + 1, 0);
   std::vector<int> amap_pos;
@@ -216,126 +260,97 @@ void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const Fron
       amap_ptr[g + 1] = (int64_t)amap_pos.size();
     }
   }
-  // per-row front id and local position; extend-add sources of every row
-  std::vector<int> row_front(rowoff[nf]), row_local(rowoff[nf]);
-  for (int g = 0; g < nf; ++g)
-    for (int r = 0; r < f[g]; ++r) {
-      row_front[rowoff[g] + r] = g;
-      row_local[rowoff[g] + r] = r;
-    }
-  std::vector<std::pair<int64_t, int64_t>> contrib;  // (parent row, child update row), child-list order
+  // child update rows landing on every front row, in child order (the elimination trees are binary)
+  std::vector<int2> csrc(rowoff[nf], make_int2(-1, -1));
   for (int g = 0; g < nf; ++g)
     for (int q = child_ptr[g]; q < child_ptr[g + 1]; ++q) {
       const int ch = child_idx[q];
       for (int a = 0; a < f[ch] - k[ch]; ++a) {
         const int64_t cr = rowoff[ch] + k[ch] + a;
-        contrib.push_back({rowoff[g] + cmap[cr], cr});
+        int2& d = csrc[rowoff[g] + cmap[cr]];
+        if (d.y >= 0) throw HzError{HZ_EINTERNAL, "front with more than two children"};
+        (d.x < 0 ? d.x : d.y) = (int)cr;
       }
     }
-  std::stable_sort(contrib.begin(), contrib.end(),
-                   [](const std::pair<int64_t, int64_t>& x, const std::pair<int64_t, int64_t>& y) {
-                     return x.first < y.first;
-                   });
-  std::vector<int64_t> cptr(rowoff[nf] + 1, 0);
-  std::vector<int> cidx(contrib.size());
-  for (size_t q = 0; q < contrib.size(); ++q) {
-    cptr[contrib[q].first + 1]++;
-    cidx[q] = (int)contrib[q].second;
+  // sweep tasks
+  std::vector<SweepTask> ftasks, btasks;
+  info.ftask_ptr.assign(1, 0);
+  info.btask_ptr.assign(1, 0);
+  info.fbrows.assign(maxh + 1, 0);
+  info.bbrows.assign(maxh + 1, 0);
+  info.fgroups.assign(maxh + 1, 0);
+  info.bgroups.assign(maxh + 1, 0);
+  for (int l = 0; l <= maxh; ++l) {
+    const int* list = level_list.data() + info.level_ptr[l];
+    const int count = info.level_ptr[l + 1] - info.level_ptr[l];
+    level_tasks(true, fp32, list, count, k, f, rowoff, Moff, Doff, ftasks, info.fbrows[l], info.fgroups[l]);
+    level_tasks(false, fp32, list, count, k, f, rowoff, MToff, Doff, btasks, info.bbrows[l], info.bgroups[l]);
+    info.ftask_ptr.push_back((int)ftasks.size());
+    info.btask_ptr.push_back((int)btasks.size());
   }
-  for (int64_t r = 0; r < rowoff[nf]; ++r) cptr[r + 1] += cptr[r];
-  // sweep tiles: (front, first output row, first reduction index, partial slot)
-  // and row blocks (front, first output row, tiles, first slot); slots restart
-  // at 0 on every level
-  std::vector<int4> ftiles, frb, btiles, brb;
-  info.ftile_ptr.assign(1, 0);
-  info.btile_ptr.assign(1, 0);
-  info.frb_ptr.assign(1, 0);
-  info.brb_ptr.assign(1, 0);
-  // tensor-core mode: eligible tiles go to the tcgen05 kernel with their factor
+  // tensor-core form: tiles (front, first output row, first reduction index, partial slot) and row
+  // blocks (front, first output row, tiles, first slot); slots restart at 0 on every level. A row block
+  // covered by a single tile finishes inside the tile (slot -1); the others sum their partial tiles in
+  // k_mf_reduce. A front without pivots (k = 0) still passes its children's updates on: its row blocks
+  // get one tile with an empty reduction. Eligible tiles go to the tcgen05 kernel with their factor
   // block packed (TF32 planes, K-major core matrices), the rest to the SIMT kernel
-  std::vector<int4> fs, bsl, ftc, btc;
+  std::vector<int4> frb, brb, fs, bsl, ftc, btc;
   std::vector<int64_t> ftc_off, btc_off;
-  int64_t tc_bytes = 0;
-  info.fs_ptr.assign(1, 0);
-  info.bs_ptr.assign(1, 0);
-  info.ftc_ptr.assign(1, 0);
-  info.btc_ptr.assign(1, 0);
-  auto classify = [&](bool fwd, const int4& tile) {
-    const int g = tile.x, r0 = tile.y, c0 = tile.z;
-    const int nout = fwd ? f[g] : k[g];
-    const int kend = fwd ? (r0 < k[g] ? std::min(k[g], r0 + MF_TILE_ROWS) : k[g]) : f[g];
-    const int kbeg = fwd ? c0 : std::max(c0, r0);
-    const int kstop = std::min(kend, c0 + MF_TILE_K);
-    const int nr = std::min(MF_TILE_ROWS, nout - r0), nk = kstop - kbeg;
-    if (tc && nr >= TC_MIN_ROWS && nk >= TC_MIN_K) {
-      (fwd ? ftc : btc).push_back(tile);
-      (fwd ? ftc_off : btc_off).push_back(tc_bytes);
-      tc_bytes += tc_tile_bytes(nr, nk);
-    } else {
-      (fwd ? fs : bsl).push_back(tile);
-    }
-  };
-  info.fwd_cmacs.assign(maxh + 1, 0.0);
-  info.fhalf.assign(maxh + 1, 1);
-  info.bhalf.assign(maxh + 1, 1);
-  info.bwd_cmacs.assign(maxh + 1, 0.0);
-  int64_t max_slots = 1;
-  for (int l = 0; l <= maxh; ++l) {
-    int fslot = 0, bslot = 0;
-    for (int q = info.level_ptr[l]; q < info.level_ptr[l + 1]; ++q) {
-      const int g = level_list[q];
-      // a row block covered by a single tile finishes inside the tile (slot
-      // -1); the others sum their partial tiles in k_mf_reduce. A front
-      // without pivots (k = 0) still passes its children's updates on: its
-      // row blocks get one tile with an empty reduction
-      for (int r0 = 0; r0 < f[g]; r0 += MF_TILE_ROWS) {
-        if (f[g] - r0 > 64) info.fhalf[l] = 0;
-        const int kend = r0 < k[g] ? std::min(k[g], r0 + MF_TILE_ROWS) : k[g];
-        const int nk = (kend + MF_TILE_K - 1) / MF_TILE_K;
-        if (nk <= 1) {
-          ftiles.push_back(make_int4(g, r0, 0, -1));
-          classify(true, ftiles.back());
-          continue;
+  int64_t tc_bytes = 0, max_slots = 1;
+  if (tc) {
+    for (auto* p : {&info.frb_ptr, &info.brb_ptr, &info.fs_ptr, &info.bs_ptr, &info.ftc_ptr, &info.btc_ptr})
+      p->assign(1, 0);
+    info.fhalf.assign(maxh + 1, 1);
+    info.bhalf.assign(maxh + 1, 1);
+    auto classify = [&](bool fwd, const int4& tile) {
+      const int g = tile.x, r0 = tile.y, c0 = tile.z;
+      const int nout = fwd ? f[g] : k[g];
+      const int kend = fwd ? (r0 < k[g] ? std::min(k[g], r0 + MF_TILE_ROWS) : k[g]) : f[g];
+      const int kbeg = fwd ? c0 : std::max(c0, r0);
+      const int kstop = std::min(kend, c0 + MF_TILE_K);
+      const int nr = std::min(MF_TILE_ROWS, nout - r0), nk = kstop - kbeg;
+      if (nr >= TC_MIN_ROWS && nk >= TC_MIN_K) {
+        (fwd ? ftc : btc).push_back(tile);
+        (fwd ? ftc_off : btc_off).push_back(tc_bytes);
+        tc_bytes += tc_tile_bytes(nr, nk);
+      } else {
+        (fwd ? fs : bsl).push_back(tile);
+      }
+    };
+    for (int l = 0; l <= maxh; ++l) {
+      int fslot = 0, bslot = 0;
+      for (int q = info.level_ptr[l]; q < info.level_ptr[l + 1]; ++q) {
+        const int g = level_list[q];
+        for (int r0 = 0; r0 < f[g]; r0 += MF_TILE_ROWS) {
+          if (f[g] - r0 > 64) info.fhalf[l] = 0;
+          const int kend = r0 < k[g] ? std::min(k[g], r0 + MF_TILE_ROWS) : k[g];
+          const int nk = (kend + MF_TILE_K - 1) / MF_TILE_K;
+          if (nk <= 1) {
+            classify(true, make_int4(g, r0, 0, -1));
+            continue;
+          }
+          frb.push_back(make_int4(g, r0, nk, fslot));
+          for (int c0 = 0; c0 < kend; c0 += MF_TILE_K) classify(true, make_int4(g, r0, c0, fslot++));
         }
-        frb.push_back(make_int4(g, r0, nk, fslot));
-        for (int c0 = 0; c0 < kend; c0 += MF_TILE_K) {
-          ftiles.push_back(make_int4(g, r0, c0, fslot++));
-          classify(true, ftiles.back());
+        for (int j0 = 0; j0 < k[g]; j0 += MF_TILE_ROWS) {
+          if (k[g] - j0 > 64) info.bhalf[l] = 0;
+          const int nk = (f[g] - j0 + MF_TILE_K - 1) / MF_TILE_K;
+          if (nk == 1) {
+            classify(false, make_int4(g, j0, j0, -1));
+            continue;
+          }
+          brb.push_back(make_int4(g, j0, nk, bslot));
+          for (int c0 = j0; c0 < f[g]; c0 += MF_TILE_K) classify(false, make_int4(g, j0, c0, bslot++));
         }
       }
-      for (int j0 = 0; j0 < k[g]; j0 += MF_TILE_ROWS) {
-        if (k[g] - j0 > 64) info.bhalf[l] = 0;
-        const int nk = (f[g] - j0 + MF_TILE_K - 1) / MF_TILE_K;
-        if (nk == 1) {
-          btiles.push_back(make_int4(g, j0, j0, -1));
-          classify(false, btiles.back());
-          continue;
-        }
-        brb.push_back(make_int4(g, j0, nk, bslot));
-        for (int c0 = j0; c0 < f[g]; c0 += MF_TILE_K) {
-          btiles.push_back(make_int4(g, j0, c0, bslot++));
-          classify(false, btiles.back());
-        }
-      }
-      const double kk = k[g], mm = f[g] - k[g];
-      info.fwd_cmacs[l] += kk * (kk + 1) / 2 + kk * mm;
-      info.bwd_cmacs[l] += kk * (kk + 1) / 2 + kk * mm;
+      max_slots = std::max<int64_t>(max_slots, std::max(fslot, bslot));
+      info.frb_ptr.push_back((int)frb.size());
+      info.brb_ptr.push_back((int)brb.size());
+      info.fs_ptr.push_back((int)fs.size());
+      info.bs_ptr.push_back((int)bsl.size());
+      info.ftc_ptr.push_back((int)ftc.size());
+      info.btc_ptr.push_back((int)btc.size());
     }
-    max_slots = std::max<int64_t>(max_slots, std::max(fslot, bslot));
-    info.ftile_ptr.push_back((int)ftiles.size());
-    info.btile_ptr.push_back((int)btiles.size());
-    info.frb_ptr.push_back((int)frb.size());
-    info.brb_ptr.push_back((int)brb.size());
-    info.fs_ptr.push_back((int)fs.size());
-    info.bs_ptr.push_back((int)bsl.size());
-    info.ftc_ptr.push_back((int)ftc.size());
-    info.btc_ptr.push_back((int)btc.size());
-  }
-  info.level_row.assign(maxh + 2, 0);
-  for (int l = 0; l <= maxh; ++l) {
-    int64_t e = info.level_row[l];
-    for (int q = info.level_ptr[l]; q < info.level_ptr[l + 1]; ++q) e += f[level_list[q]];
-    info.level_row[l + 1] = e;
   }
   mf.nfronts = nf;
   mf.nlevels = info.nlevels;
@@ -344,98 +359,51 @@ void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const Fron
   mf.F_total = Foff[nf];
   mf.amap_total = (int64_t)amap_pos.size();
   mf.level_ptr_h = info.level_ptr.data();
-  mf.ftile_ptr_h = info.ftile_ptr.data();
-  mf.fhalf_h = info.fhalf.data();
-  mf.bhalf_h = info.bhalf.data();
-  mf.btile_ptr_h = info.btile_ptr.data();
-  mf.frb_ptr_h = info.frb_ptr.data();
-  mf.brb_ptr_h = info.brb_ptr.data();
-  mf.level_row_h = info.level_row.data();
-  mf.max_slots = max_slots;
+  mf.ftask_ptr_h = info.ftask_ptr.data();
+  mf.btask_ptr_h = info.btask_ptr.data();
+  mf.fbrows_h = info.fbrows.data();
+  mf.bbrows_h = info.bbrows.data();
+  mf.fgroups_h = info.fgroups.data();
+  mf.bgroups_h = info.bgroups.data();
+  mf.ftasks = pool.upload(ftasks, st);
+  mf.btasks = pool.upload(btasks, st);
+  mf.csrc = pool.upload(csrc, st);
   if (persistent) {
-    // the same tiles renumbered for one launch per sweep: slots unique over all levels, the
-    // backward tiles ordered from the roots down
-    std::vector<int4> ptf, ptb, prbf, prbb;
-    std::vector<int> srf, srb, nrbf(nf, 0), nrbb(nf, 0), nch(nf);
-    for (int g = 0; g < nf; ++g) nch[g] = child_ptr[g + 1] - child_ptr[g];
-    auto renumber = [&](const std::vector<int4>& tl, const std::vector<int>& tptr, bool fwd, std::vector<int4>& out,
-                        std::vector<int4>& rbs, std::vector<int>& slot_rb, std::vector<int>& nrb) {
-      for (int li = 0; li <= maxh; ++li) {
-        const int l = fwd ? li : maxh - li;
-        // within a level, tiles of one row block are adjacent (built that way above)
-        for (int q = tptr[l]; q < tptr[l + 1]; ++q) {
-          int4 t = tl[q];
-          if (t.w < 0) {
-            out.push_back(t);
-            nrb[t.x]++;
-            continue;
-          }
-          const bool first = out.empty() || out.back().w < 0 || out.back().x != t.x || out.back().y != t.y;
-          if (first) {
-            rbs.push_back(make_int4(t.x, t.y, 0, (int)slot_rb.size()));
-            nrb[t.x]++;
-          }
-          rbs.back().z++;
-          t.w = (int)slot_rb.size();
-          slot_rb.push_back((int)rbs.size() - 1);
-          out.push_back(t);
-        }
-      }
-    };
-    renumber(ftiles, info.ftile_ptr, true, ptf, prbf, srf, nrbf);
-    renumber(btiles, info.btile_ptr, false, ptb, prbb, srb, nrbb);
-    // forward: a front waits for its children that have rows (a child without rows has no update
-    // rows either and contributes nothing); backward: a front waits for its nearest ancestor with
-    // pivots, which finishes only after all of its own ancestors
-    std::vector<int> bdep(nf, -1);
+    // the same tasks, the backward ones from the roots down. Forward: a front waits for its children
+    // that have rows (a child without rows has no update rows either and contributes nothing);
+    // backward: a front waits for its nearest ancestor with pivots, which finishes only after all of
+    // its own ancestors
+    std::vector<SweepTask> top;
+    for (int l = maxh; l >= 0; --l)
+      top.insert(top.end(), btasks.begin() + info.btask_ptr[l], btasks.begin() + info.btask_ptr[l + 1]);
+    std::vector<int> nft(nf, 0), nbt(nf, 0), nch(nf, 0), bdep(nf, -1);
+    for (const SweepTask& t : ftasks) nft[t.front]++;
+    for (const SweepTask& t : btasks) nbt[t.front]++;
     for (int g = 0; g < nf; ++g) {
-      nch[g] = 0;
-      for (int q = child_ptr[g]; q < child_ptr[g + 1]; ++q) nch[g] += nrbf[child_idx[q]] > 0;
+      for (int q = child_ptr[g]; q < child_ptr[g + 1]; ++q) nch[g] += nft[child_idx[q]] > 0;
       int a = parent[g];
-      while (a >= 0 && nrbb[a] == 0) a = parent[a];
+      while (a >= 0 && nbt[a] == 0) a = parent[a];
       bdep[g] = a;
     }
     mf.persistent = 1;
-    mf.pt_nf = (int)ptf.size();
-    mf.pt_nb = (int)ptb.size();
-    mf.prb_nf = (int)prbf.size();
-    mf.prb_nb = (int)prbb.size();
-    mf.ptf = pool.upload(ptf, st);
-    mf.ptb = pool.upload(ptb, st);
-    mf.slot_rb_f = pool.upload(srf, st);
-    mf.slot_rb_b = pool.upload(srb, st);
-    mf.prb_f = pool.upload(prbf, st);
-    mf.prb_b = pool.upload(prbb, st);
-    mf.nrb_f = pool.upload(nrbf, st);
-    mf.nrb_b = pool.upload(nrbb, st);
+    mf.btasks_top = pool.upload(top, st);
+    mf.front_ftasks = pool.upload(nft, st);
+    mf.front_btasks = pool.upload(nbt, st);
     mf.parent = pool.upload(parent, st);
     mf.bdep = pool.upload(bdep, st);
     mf.nchild = pool.upload(nch, st);
-    mf.cnt_n = 1 + std::max(mf.prb_nf, mf.prb_nb) + 2 * nf;
-    mf.cnt = pool.alloc<int>(mf.cnt_n);
-    mf.pslots = std::max<int64_t>(1, std::max(srf.size(), srb.size()));
+    mf.cnt = pool.alloc<int>(1 + 2 * (size_t)nf);
     mf.sw_err = pool.alloc<int>(1);
     CK(cudaMemsetAsync(mf.sw_err, 0, sizeof(int), st));
   }
-  mf.frb = pool.upload(frb, st);
-  mf.brb = pool.upload(brb, st);
-  mf.row_front = pool.upload(row_front, st);
-  mf.row_local = pool.upload(row_local, st);
-  mf.cptr = pool.upload(cptr, st);
-  mf.cidx = pool.upload(cidx, st);
-  mf.cidx_n = (int64_t)cidx.size();
-  mf.ftiles_n = (int64_t)ftiles.size();
-  mf.btiles_n = (int64_t)btiles.size();
   mf.fp32 = fp32 ? 1 : 0;
-  mf.M_total = Moff[nf];
   mf.D_total = Doff[nf];
-  mf.ftiles = pool.upload(ftiles, st);
-  mf.btiles = pool.upload(btiles, st);
   mf.Moff = pool.upload(Moff, st);
+  mf.MToff = pool.upload(MToff, st);
   mf.Doff = pool.upload(Doff, st);
   const size_t esz = fp32 ? sizeof(float2) : sizeof(double2);
   mf.M = pool.alloc<char>(Moff[nf] * esz);
-  mf.MT = pool.alloc<char>(Moff[nf] * esz);
+  mf.MT = pool.alloc<char>(MToff[nf] * esz);
   mf.Dinv = pool.alloc<char>(Doff[nf] * esz);
   mf.level_list = pool.upload(level_list, st);
   mf.k = pool.upload(k, st);
@@ -522,6 +490,13 @@ void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const Fron
   CK(cudaMemsetAsync(mf.perturbed, 0, sizeof(int), st));
   mf.tc = tc ? 1 : 0;
   if (tc) {
+    mf.frb_ptr_h = info.frb_ptr.data();
+    mf.brb_ptr_h = info.brb_ptr.data();
+    mf.fhalf_h = info.fhalf.data();
+    mf.bhalf_h = info.bhalf.data();
+    mf.frb = pool.upload(frb, st);
+    mf.brb = pool.upload(brb, st);
+    mf.max_slots = max_slots;
     mf.fs_ptr_h = info.fs_ptr.data();
     mf.bs_ptr_h = info.bs_ptr.data();
     mf.ftc_ptr_h = info.ftc_ptr.data();
@@ -863,9 +838,10 @@ void ensure_workspace(hz_ctx* c, int s) {
   c->Q = p.alloc<double2>(n * s);
   c->U = p.alloc<double2>(n * s);
   const size_t ef = c->lf.mf.fp32 ? sizeof(float2) : sizeof(double2);
-  c->Xsub = (double2*)p.alloc<char>(c->lf.sub_rows * s * ef);
-  c->lf.mf.Wout = p.alloc<char>(c->lf.mf.rows_total * s * ef);
-  c->lf.mf.P = p.alloc<char>((size_t)std::max(c->lf.mf.max_slots, c->lf.mf.pslots) * MF_TILE_ROWS * s * ef);
+  const int cols = sweep_cols(s);
+  c->Xsub = (double2*)p.alloc<char>(c->lf.sub_rows * cols * ef);
+  c->lf.mf.Wout = p.alloc<char>(c->lf.mf.rows_total * cols * ef);
+  if (c->lf.mf.tc) c->lf.mf.P = p.alloc<char>((size_t)c->lf.mf.max_slots * MF_TILE_ROWS * cols * ef);
   c->lf.mf.s_cap = s;
   // double-float Arnoldi for the outer space unless block FGMRES or recycling (which read W in FP64)
   alloc_krylov(c->Kout, n, s, c->opt.restart, p, false,
@@ -913,9 +889,9 @@ void ensure_workspace(hz_ctx* c, int s) {
     c->rH = p.alloc<double2>(nh * s);
     c->yH = p.alloc<double2>(nh * s);
     const size_t ec = c->lc.mf.fp32 ? sizeof(float2) : sizeof(double2);
-    c->XsubH = (double2*)p.alloc<char>(c->lc.sub_rows * s * ec);
-    c->lc.mf.Wout = p.alloc<char>(c->lc.mf.rows_total * s * ec);
-    c->lc.mf.P = p.alloc<char>((size_t)std::max(c->lc.mf.max_slots, c->lc.mf.pslots) * MF_TILE_ROWS * s * ec);
+    c->XsubH = (double2*)p.alloc<char>(c->lc.sub_rows * cols * ec);
+    c->lc.mf.Wout = p.alloc<char>(c->lc.mf.rows_total * cols * ec);
+    if (c->lc.mf.tc) c->lc.mf.P = p.alloc<char>((size_t)c->lc.mf.max_slots * MF_TILE_ROWS * cols * ec);
     c->lc.mf.s_cap = s;
     if (c->opt.coarse_mode == HZ_COARSE_GMRES) {
       alloc_krylov(c->Kin, nh, s, std::max(1, c->opt.coarse_inner_its), p, c->coarse32, c->df);
@@ -972,7 +948,7 @@ void apply_oras(LevelDev& L, const double2* V, double2* Zout, const double2* Qad
   const double fflops = 8.0 * s * 2.0 * L.info.factor_entries;
   int p0 = prof ? prof->begin(PH_RESTRICT, st) : -1;
   if (L.mf.fp32)
-    gather_rows_f32(L.mf.gidx, L.sub_rows, V, (float2*)Xsub, s, st);
+    gather_rows(L.mf.gidx, L.sub_rows, V, (float2*)Xsub, s, st);
   else
     gather_rows(L.mf.gidx, L.sub_rows, V, Xsub, s, st);
   if (prof) prof->end(p0, st, 0.0, 0.0);
@@ -981,7 +957,7 @@ void apply_oras(LevelDev& L, const double2* V, double2* Zout, const double2* Qad
   if (prof) prof->end(p1, st, fflops, fbytes);
   int p2 = prof ? prof->begin(PH_RESTRICT, st) : -1;
   if (L.mf.fp32)
-    scatter_owned_f32(L.mf.own, L.n, (const float2*)Xsub, Qadd, Zout, s, st);
+    scatter_owned(L.mf.own, L.n, (const float2*)Xsub, Qadd, Zout, s, st);
   else
     scatter_owned(L.mf.own, L.n, Xsub, Qadd, Zout, s, st);
   if (prof) prof->end(p2, st, 0.0, rbytes);
@@ -1009,9 +985,9 @@ void coarse_solve(hz_ctx* c, const double2* rH, double2* yH, int s) {
     CK(cudaMemsetAsync(c->yH32, 0, vs * sizeof(float2), st));
     krylov_start(K, c->rH32, st);
     for (int j = 0; j < K.m; ++j) {
-      gather_rows_ff(L.mf.gidx, L.sub_rows, V + j * vs, Xs, s, st);
+      gather_rows(L.mf.gidx, L.sub_rows, V + j * vs, Xs, s, st);
       mf_solve(L.mf, Xs, s, st);
-      scatter_owned_ff(L.mf.own, L.n, Xs, Zk + j * vs, s, st);
+      scatter_owned(L.mf.own, L.n, Xs, (const float2*)nullptr, Zk + j * vs, s, st);
       spmm_split_f32(c->E, Zk + j * vs, (float2*)K.W, s, st);
       krylov_arnoldi(K, j, st);
     }
@@ -1130,14 +1106,14 @@ void apply_prec(hz_ctx* c, const double2* V, double2* Zout, int s) {
                 6.0 * (c->A.nnz_re + c->A.nnz_im) + 16.0 * (n + 1) + 24.0 * n * s);
     LevelDev& L = c->lf;
     int p0 = c->prof.begin(PH_RESTRICT, st);
-    gather_rows_ff(L.mf.gidx, L.sub_rows, c->t32, (float2*)c->Xsub, s, st);
+    gather_rows(L.mf.gidx, L.sub_rows, c->t32, (float2*)c->Xsub, s, st);
     c->prof.end(p0, st, 0.0, 0.0);
     int p1 = c->prof.begin(PH_FRONTS, st);
     run_graph(gf, s, st, [&]() { mf_solve(L.mf, c->Xsub, s, st); });
     c->prof.end(p1, st, 8.0 * s * 2.0 * L.info.factor_entries,
                 8.0 * 2.0 * L.info.factor_entries + 2.0 * 8.0 * s * L.sub_rows);
     int p2 = c->prof.begin(PH_RESTRICT, st);
-    scatter_owned_fq(L.mf.own, L.n, (const float2*)c->Xsub, c->q32, Zout, s, st);     // z = M1^{-1} t + q
+    scatter_owned(L.mf.own, L.n, (const float2*)c->Xsub, c->q32, Zout, s, st);     // z = M1^{-1} t + q
     c->prof.end(p2, st, 0.0, 4.0 * L.sub_rows + 16.0 * L.sub_rows * s + 4.0 * L.n + 32.0 * L.n * s);
     return;
   }
@@ -1461,10 +1437,13 @@ void check_bounds(hz_ctx* c) {
     chk(lev ? "coarse R_i map" : "fine R_i map", mf.gidx, mf.nsub_rows, 1, 0, L.n);
     chk(lev ? "coarse owner map" : "fine owner map", mf.own, L.n, 1, 0, mf.nsub_rows);
     chk(lev ? "coarse front rows" : "fine front rows", mf.rows, mf.rows_total, 1, 0, mf.nsub_rows);
-    chk(lev ? "coarse extend-add sources" : "fine extend-add sources", mf.cidx, mf.cidx_n, 1, 0, mf.rows_total);
+    chk(lev ? "coarse extend-add sources" : "fine extend-add sources", mf.csrc, 2 * mf.rows_total, 1, -1, mf.rows_total);
     chk(lev ? "coarse level list" : "fine level list", mf.level_list, mf.nfronts, 1, 0, mf.nfronts);
-    chk(lev ? "coarse forward tiles" : "fine forward tiles", mf.ftiles, mf.ftiles_n, 4, 0, mf.nfronts);
-    chk(lev ? "coarse backward tiles" : "fine backward tiles", mf.btiles, mf.btiles_n, 4, 0, mf.nfronts);
+    const int front = offsetof(SweepTask, front) / sizeof(int), words = sizeof(SweepTask) / sizeof(int);
+    chk(lev ? "coarse forward tasks" : "fine forward tasks", (const int*)mf.ftasks + front, mf.ftask_ptr_h[mf.nlevels],
+        words, 0, mf.nfronts);
+    chk(lev ? "coarse backward tasks" : "fine backward tasks", (const int*)mf.btasks + front,
+        mf.btask_ptr_h[mf.nlevels], words, 0, mf.nfronts);
   }
   if (c->has_coarse) {
     chk_csr("E columns", c->E.col_re, c->E.nnz_re, c->E.ncols);

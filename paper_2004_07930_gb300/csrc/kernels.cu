@@ -114,35 +114,79 @@ void spmm_real(int64_t nrows, const int64_t* rp, const int32_t* col, const doubl
 // Restriction R_i (gather, K2) and Boolean partition-of-unity prolongation
 // sum_i R_i^T D_i (each dof read from its owning subdomain copy, K3)
 // ---------------------------------------------------------------------------
-__global__ void k_gather_rows(const int* __restrict__ idx, int64_t nrows, const double2* __restrict__ X,
-                              double2* __restrict__ Y, int s) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
+// Threads are (column, row) pairs, so that no index is divided by the block
+// width; a sub-vector row has `cols` entries, those from s on zero.
+template <typename In, typename Out>
+__global__ void k_gather(const int* __restrict__ idx, int64_t nrows, const In* __restrict__ X, Out* __restrict__ Y, int s,
+                         int cols) {
+  const int64_t r = blockIdx.x * (int64_t)blockDim.y + threadIdx.y;
+  const int c = threadIdx.x;
   if (r >= nrows) return;
-  int c = (int)(g - r * s);
-  Y[g] = X[(int64_t)idx[r] * s + c];
+  Out y;
+  y.x = y.y = 0;
+  if (c < s) {
+    const In x = X[(int64_t)idx[r] * s + c];
+    y.x = (decltype(y.x))x.x;
+    y.y = (decltype(y.y))x.y;
+  }
+  Y[r * cols + c] = y;
+}
+
+template <typename In, typename Q, typename Out>
+__global__ void k_scatter(const int* __restrict__ own, int64_t n, const In* __restrict__ Xsub, const Q* __restrict__ Qb,
+                          Out* __restrict__ Z, int s, int cols) {
+  const int64_t r = blockIdx.x * (int64_t)blockDim.y + threadIdx.y;
+  const int c = threadIdx.x;
+  if (r >= n) return;
+  const In x = Xsub[(int64_t)own[r] * cols + c];
+  Out z;
+  z.x = x.x;
+  z.y = x.y;
+  if (Qb) {
+    const Q q = Qb[r * s + c];
+    z.x += (decltype(z.x))q.x;
+    z.y += (decltype(z.y))q.y;
+  }
+  Z[r * s + c] = z;
+}
+
+template <typename In, typename Out>
+static void gather_t(const int* idx, int64_t nrows, const In* X, Out* Y, int s, cudaStream_t st) {
+  if (nrows * s == 0) return;
+  const int cols = sweep_cols(s);
+  const dim3 b(cols, std::max(1, 256 / cols));
+  { k_gather<<<grid_for(nrows, b.y), b, 0, st>>>(idx, nrows, X, Y, s, cols); count_launch(); }
+}
+template <typename In, typename Q, typename Out>
+static void scatter_t(const int* own, int64_t n, const In* Xsub, const Q* Qb, Out* Z, int s, cudaStream_t st) {
+  if (n * s == 0) return;
+  const dim3 b(s, std::max(1, 256 / s));
+  { k_scatter<<<grid_for(n, b.y), b, 0, st>>>(own, n, Xsub, Qb, Z, s, sweep_cols(s)); count_launch(); }
 }
 
 void gather_rows(const int* idx, int64_t nrows, const double2* X, double2* Y, int s, cudaStream_t st) {
-  if (nrows * s == 0) return;
-  { k_gather_rows<<<grid_for(nrows * s, 256), 256, 0, st>>>(idx, nrows, X, Y, s); count_launch(); }
+  gather_t(idx, nrows, X, Y, s, st);
 }
-
-__global__ void k_scatter_owned(const int* __restrict__ own, int64_t n, const double2* __restrict__ Xsub,
-                                const double2* __restrict__ Q, double2* __restrict__ Z, int s) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  if (r >= n) return;
-  int c = (int)(g - r * s);
-  double2 v = Xsub[(int64_t)own[r] * s + c];
-  if (Q) v = cadd(v, Q[g]);
-  Z[g] = v;
+void gather_rows(const int* idx, int64_t nrows, const double2* X, float2* Y, int s, cudaStream_t st) {
+  gather_t(idx, nrows, X, Y, s, st);
 }
-
+void gather_rows(const int* idx, int64_t nrows, const float2* X, float2* Y, int s, cudaStream_t st) {
+  gather_t(idx, nrows, X, Y, s, st);
+}
 void scatter_owned(const int* own, int64_t n, const double2* Xsub, const double2* Q, double2* Z, int s,
                    cudaStream_t st) {
-  if (n * s == 0) return;
-  { k_scatter_owned<<<grid_for(n * s, 256), 256, 0, st>>>(own, n, Xsub, Q, Z, s); count_launch(); }
+  scatter_t(own, n, Xsub, Q, Z, s, st);
+}
+void scatter_owned(const int* own, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
+                   cudaStream_t st) {
+  scatter_t(own, n, Xsub, Q, Z, s, st);
+}
+void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
+                   cudaStream_t st) {
+  scatter_t(own, n, Xsub, Q, Z, s, st);
+}
+void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st) {
+  scatter_t(own, n, Xsub, Q, Z, s, st);
 }
 
 __global__ void k_zero(double2* X, int64_t count) {

@@ -29,39 +29,98 @@ struct DevSplitCsr {
   float2* val_im_df = nullptr;
 };
 
+// Grouped factor layout. The rows of X_t (f x k, unit lower trapezoidal) and
+// of X_t^T are cut into groups of MF_GR; a group stores [reduction index][row]
+// with its row count padded to 4 (the front's last group only), without the
+// structural zeros: group g of X_t the columns below min(k, MF_GR (g + 1)),
+// group g of X_t^T the columns from MF_GR g on. Every group is contiguous and
+// starts on a multiple of 32 bytes. In FP32 two neighbouring rows share 16
+// bytes, (re, re, im, im), the operand pairs of the packed FP32 multiply-add.
+constexpr int MF_GR = 16;      // rows per group
+constexpr int MF_CHUNK = 128;  // reduction indices summed before the running total takes them
+constexpr int MF_RES = 256;    // longest reduction whose input rows a sweep task keeps in shared memory
+__host__ __device__ inline int mf_group_rows(int nout, int g) {  // padded rows of group g of nout rows
+  const int nr = nout - MF_GR * g;
+  return nr >= MF_GR ? MF_GR : (nr + 3) & ~3;
+}
+// entries stored before group g
+__host__ __device__ inline int64_t mf_fwd_before(int k, int g) {
+  const int64_t full = k / MF_GR, t = g < full ? g : full;  // groups with all their MF_GR (i + 1) columns
+  return MF_GR * MF_GR / 2 * t * (t + 1) + (g - t) * MF_GR * (int64_t)k;
+}
+__host__ __device__ inline int64_t mf_bwd_before(int f, int g) {
+  return MF_GR * (int64_t)f * g - MF_GR * MF_GR / 2 * (int64_t)g * (g - 1);
+}
+// entries of a front
+__host__ __device__ inline int64_t mf_fwd_size(int f, int k) {
+  const int g = (f - 1) / MF_GR, len = k < MF_GR * (g + 1) ? k : MF_GR * (g + 1);
+  return f > 0 ? mf_fwd_before(k, g) + (int64_t)mf_group_rows(f, g) * len : 0;
+}
+__host__ __device__ inline int64_t mf_bwd_size(int f, int k) {
+  const int g = (k - 1) / MF_GR;
+  return k > 0 ? mf_bwd_before(f, g) + (int64_t)mf_group_rows(k, g) * (f - MF_GR * g) : 0;
+}
+// entry of row `rl` of a group at reduction index `i` (both counted inside the
+// group), the group's entries at `g` with `nrp` padded rows
+__device__ inline void mf_put(double2* g, int nrp, int i, int rl, double2 v) { g[(int64_t)i * nrp + rl] = v; }
+__device__ inline void mf_put(float2* g, int nrp, int i, int rl, float2 v) {
+  float* p = reinterpret_cast<float*>(g + (int64_t)i * nrp) + (rl >> 1) * 4 + (rl & 1);
+  p[0] = v.x;
+  p[2] = v.y;
+}
+__device__ inline float2 mf_get(const float2* g, int nrp, int i, int rl) {
+  const float* p = reinterpret_cast<const float*>(g + (int64_t)i * nrp) + (rl >> 1) * 4 + (rl & 1);
+  return make_float2(__ldg(p), __ldg(p + 2));
+}
+// X_t[r][c] and X_t^T[c][r] for c / MF_GR <= r / MF_GR (the other entries are
+// structural zeros of both sweeps and are not stored)
+template <typename V>
+__device__ inline void mf_store(V* Mt, V* MTt, int f, int k, int r, int c, V v) {
+  const int gr = r / MF_GR, gc = c / MF_GR;
+  if (gc > gr) return;
+  mf_put(Mt + mf_fwd_before(k, gr), mf_group_rows(f, gr), c, r - MF_GR * gr, v);
+  mf_put(MTt + mf_bwd_before(f, gc), mf_group_rows(k, gc), r - MF_GR * gc, c - MF_GR * gc, v);
+}
+
+// One CTA's share of a sweep level: groups [g0, g0 + ng) of a front, with
+// the front's data beside it so that no lookup precedes the first loads.
+struct alignas(16) SweepTask {
+  int64_t m;      // offset of the front's factor (X_t or X_t^T)
+  int64_t row;    // first front row
+  int32_t d;      // offset of 1/D
+  int32_t front;
+  uint16_t k, f;
+  uint16_t g0, ng;
+};
+static_assert(sizeof(SweepTask) == 32, "sweep tasks are read as two 16-byte words");
+
 // Multifrontal factors of a batch of local matrices, grouped by tree height.
-// Factor storage per front t: X_t (f x k, column-major) = first k columns of
-// [[L11,0],[L21,I]]^{-1}, and 1/D (k); FP64 or FP32 (mixed form).
+// Factor storage per front t: X_t (f x k) = first k columns of
+// [[L11,0],[L21,I]]^{-1}, in the grouped layout above, and 1/D (k); FP64 or
+// FP32 (mixed form).
 struct DevMF {
-  int64_t nfronts = 0, nsub_rows = 0, rows_total = 0, F_total = 0, amap_total = 0, M_total = 0, D_total = 0;
+  int64_t nfronts = 0, nsub_rows = 0, rows_total = 0, F_total = 0, amap_total = 0, D_total = 0;
   int nlevels = 0;
   int max_f = 0;
   int fp32 = 0;
   int* level_ptr_h = nullptr;   // host [nlevels+1]
-  int* ftile_ptr_h = nullptr;   // host [nlevels+1] forward tiles per level
-  const char* fhalf_h = nullptr;  // host [nlevels]: every forward tile of the level has <= 64 output rows
-  const char* bhalf_h = nullptr;  // host [nlevels]: the same for the backward tiles
-  int* btile_ptr_h = nullptr;   // host [nlevels+1] backward tiles per level
   int* level_list = nullptr;    // device [nfronts] front ids ordered by height
-  int* frb_ptr_h = nullptr;     // host [nlevels+1] forward row blocks per level
-  int* brb_ptr_h = nullptr;     // host [nlevels+1] backward row blocks per level
-  int64_t* level_row_h = nullptr;  // host [nlevels+1] first front row of each level
-  int64_t max_slots = 0;        // partial-result slots of the largest level
-  int4* ftiles = nullptr;       // forward tiles (front, first row, first column, slot)
-  int4* btiles = nullptr;       // backward tiles (front, first pivot, first row, slot)
-  int4* frb = nullptr;          // forward row blocks (front, first row, tiles, first slot)
-  int4* brb = nullptr;          // backward row blocks
-  int* row_front = nullptr;     // [rows_total] front of each front row
-  int* row_local = nullptr;     // [rows_total] position inside its front
-  int64_t* cptr = nullptr;      // [rows_total+1] extend-add sources of each front row
-  int* cidx = nullptr;          // child update rows, in child order
-  int64_t cidx_n = 0;           // entries of cidx
-  int64_t ftiles_n = 0, btiles_n = 0;  // tiles of each sweep (all levels)
-  void* P = nullptr;            // partial tile results [max_slots][128][s_cap]
+  // sweep tasks (sweep.cu): runs of 16-row groups of one front, level by level, and per level the
+  // longest reduction of its tasks
+  SweepTask* ftasks = nullptr;  // forward, leaves first
+  SweepTask* btasks = nullptr;  // backward, levels in the same order as forward
+  const int* ftask_ptr_h = nullptr;  // host [nlevels+1]
+  const int* btask_ptr_h = nullptr;
+  const int* fbrows_h = nullptr;     // host [nlevels]
+  const int* bbrows_h = nullptr;
+  const int* fgroups_h = nullptr;    // host [nlevels] groups of the level
+  const int* bgroups_h = nullptr;
+  int2* csrc = nullptr;         // [rows_total] child update rows landing on each front row (-1: none), child order
   int* k = nullptr;             // pivots per front
   int* f = nullptr;             // front order k + m
   int64_t* Foff = nullptr;      // offset of the f x f front workspace (column-major)
   int64_t* Moff = nullptr;      // offset of X_t in M
+  int64_t* MToff = nullptr;     // offset of X_t^T in MT
   int64_t* Doff = nullptr;      // offset of 1/D in Dinv
   int64_t* rowoff = nullptr;    // offset of the front's row list (prefix sum of f)
   int* rows = nullptr;          // [rows_total] flat sub-vector row of each front row
@@ -89,8 +148,8 @@ struct DevMF {
   int* fi_tile_ptr_h = nullptr;   // host [steps+1]
   int64_t* fa_pan_off = nullptr;  // [big fronts] offset of each large front's scratch panel (f x FA_NB_H)
   void* fa_pan = nullptr;         // scratch panels, element type of F
-  void* M = nullptr;            // X_t factors (double2 or float2), column-major f x k
-  void* MT = nullptr;           // X_t^T, column-major k x f (backward sweep)
+  void* M = nullptr;            // X_t factors (double2 or float2), grouped layout
+  void* MT = nullptr;           // X_t^T (backward sweep), grouped layout
   void* Dinv = nullptr;         // 1/D (double2 or float2)
   void* Wout = nullptr;         // front vectors [rows_total][s_cap]: y_P and parent updates
   int s_cap = 0;
@@ -101,6 +160,16 @@ struct DevMF {
   // TC_MIN_K reduction indices run as tcgen05 MMAs (three-term TF32 split, FP32 accumulation in
   // TMEM) when the block has 9-16 columns; the others keep the SIMT kernel
   int tc = 0;                   // packed tensor-core tiles present
+  // the tile form's lists: 128-row x 128-index tiles (front, first row, first index, partial slot), the
+  // row blocks that more than one tile contributes to, and the partial results
+  const char* fhalf_h = nullptr;   // host [nlevels]: every forward tile of the level has <= 64 output rows
+  const char* bhalf_h = nullptr;
+  int* frb_ptr_h = nullptr;        // host [nlevels+1] forward row blocks per level
+  int* brb_ptr_h = nullptr;
+  int4* frb = nullptr;             // (front, first row, tiles, first slot)
+  int4* brb = nullptr;
+  int64_t max_slots = 0;           // partial-result slots of the largest level
+  void* P = nullptr;               // partial tile results [max_slots][128][s_cap]
   int* fs_ptr_h = nullptr;      // host [nlevels+1] forward SIMT tiles per level (tensor-core mode)
   int* bs_ptr_h = nullptr;      // host [nlevels+1] backward SIMT tiles per level
   int* ftc_ptr_h = nullptr;     // host [nlevels+1] forward tensor-core tiles per level
@@ -117,28 +186,17 @@ struct DevMF {
   int* tc_err = nullptr;        // device flag: a tensor-core tile gave up waiting on a barrier
   cudaStream_t side = nullptr;  // tensor-core mode: the SIMT tiles of a level run here, beside the tcgen05 tiles
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  // persistent sweeps (one launch per direction): tiles in ticket order with slots numbered over all
-  // levels, row blocks (front, first row, tiles, first slot), slot -> row block, per-front row-block
-  // counts, parent and child counts, and the counters reset before every sweep
+  // persistent sweeps (one launch per direction): tasks per front, dependencies and the counters
+  // reset before every sweep
   int persistent = 0;
-  int pt_nf = 0, pt_nb = 0;     // tiles of the forward / backward sweep
-  int prb_nf = 0, prb_nb = 0;   // row blocks with partial tiles
-  int4* ptf = nullptr;          // forward tiles, leaves first
-  int4* ptb = nullptr;          // backward tiles, roots first
-  int* slot_rb_f = nullptr;
-  int* slot_rb_b = nullptr;
-  int4* prb_f = nullptr;
-  int4* prb_b = nullptr;
-  int* nrb_f = nullptr;         // [nfronts] row blocks of each front, forward
-  int* nrb_b = nullptr;         // [nfronts] backward
+  SweepTask* btasks_top = nullptr;  // backward tasks, roots first
+  int* front_ftasks = nullptr;  // [nfronts] forward tasks of each front
+  int* front_btasks = nullptr;  // [nfronts] backward tasks
   int* parent = nullptr;        // [nfronts] parent front (-1: root)
   int* bdep = nullptr;          // [nfronts] nearest ancestor with pivots (-1: none): backward dependency
-  int* nchild = nullptr;        // [nfronts]
-  int* cnt = nullptr;           // ticket | row-block counts | front counts | ready children
-  int cnt_n = 0;
-  int64_t pslots = 0;           // partial slots of the larger sweep
+  int* nchild = nullptr;        // [nfronts] children with rows
+  int* cnt = nullptr;           // ticket | finished tasks per front | finished children per front
   int* sw_err = nullptr;        // device flag: a persistent sweep gave up waiting
-  int sweep_grid = 0;           // resident CTAs of the sweep kernel
 };
 
 // fronts of order <= FA_SMALL are factored pivot by pivot, larger ones by panels of FA_NB_H pivots
@@ -164,17 +222,27 @@ void spmm_real(int64_t nrows, const int64_t* rp, const int32_t* col, const doubl
                double2* Y, int s, cudaStream_t st);
 
 // --- restriction / prolongation ---
+// Sub-vectors have rows of sweep_cols(s) entries, the columns past s zero.
+int sweep_cols(int s);  // sweep.cu
+// Y[r][:] = X[idx[r]][:] (R_i), in the sub-vector's precision
 void gather_rows(const int* idx, int64_t nrows, const double2* X, double2* Y, int s, cudaStream_t st);
+void gather_rows(const int* idx, int64_t nrows, const double2* X, float2* Y, int s, cudaStream_t st);
+void gather_rows(const int* idx, int64_t nrows, const float2* X, float2* Y, int s, cudaStream_t st);
+// Z[r][:] = Xsub[own[r]][:] (+ Q[r][:]), in Z's precision (Q may be NULL)
 void scatter_owned(const int* own, int64_t n, const double2* Xsub, const double2* Q, double2* Z, int s,
                    cudaStream_t st);
+void scatter_owned(const int* own, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
+                   cudaStream_t st);
+void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
+                   cudaStream_t st);
+void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st);
 
 // --- multifrontal ---
 void mf_factor(DevMF& mf, double tau_abs, cudaStream_t st);
-void mf_solve(DevMF& mf, void* Xsub, int s, cudaStream_t st);  // Xsub double2 or float2 (mf.fp32)
+void mf_solve(DevMF& mf, void* Xsub, int s, cudaStream_t st);  // Xsub double2 or float2 (mf.fp32), [rows][sweep_cols(s)]
+void sweep_attrs(bool fp32);                                         // sweep.cu
+void sweep_solve(DevMF& mf, void* Xsub, int cols, cudaStream_t st);  // sweep.cu; cols = sweep_cols(s)
 bool mf_tc_usable(const DevMF& mf, int s);  // the block width runs the tensor-core sweeps
-void gather_rows_f32(const int* idx, int64_t nrows, const double2* X, float2* Y, int s, cudaStream_t st);
-void scatter_owned_f32(const int* own, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
-                       cudaStream_t st);
 
 // --- Krylov (one Krylov space per column) ---
 // Vector-typed arrays hold double2 (fp32 = 0) or float2 (fp32 = 1); the
@@ -274,10 +342,6 @@ void spmm_split_f32(const DevSplitCsr& A, const float2* X, float2* Y, int s, cud
                     const float2* B = nullptr);  // Y = A X, or B - A X
 void spmm_real_f32(int64_t nrows, const int64_t* rp, const int32_t* col, const float* val, const float2* X,
                    float2* Y, int s, cudaStream_t st);
-void scatter_owned_fq(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
-                      cudaStream_t st);
-void gather_rows_ff(const int* idx, int64_t nrows, const float2* X, float2* Y, int s, cudaStream_t st);
-void scatter_owned_ff(const int* own, int64_t n, const float2* Xsub, float2* Z, int s, cudaStream_t st);
 void cast_d2f(const double2* X, float2* Y, int64_t count, cudaStream_t st);
 void cast_f2d(const float2* X, double2* Y, int64_t count, cudaStream_t st);
 

@@ -483,8 +483,7 @@ void krylov_update(DevKrylov& K, void* X, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// FP32 coarse-level helpers (mixed form): SpMM with float values, gathers
-// and scatters between FP32 blocks, precision casts
+// FP32 coarse-level helpers (mixed form): SpMM with float values, precision casts
 // ---------------------------------------------------------------------------
 // Y = A X, or Y = B - A X when B is given (FP32 values and blocks)
 __global__ void k_spmm_split_f32(int64_t n, int s, const int64_t* __restrict__ rp_re, const int32_t* __restrict__ col_re,
@@ -545,43 +544,6 @@ __global__ void k_spmm_real_f32(int64_t n, int s, const int64_t* __restrict__ rp
 void spmm_real_f32(int64_t nrows, const int64_t* rp, const int32_t* col, const float* val, const float2* X,
                    float2* Y, int s, cudaStream_t st) {
   if (nrows * s) { k_spmm_real_f32<<<grid_for(nrows * s, 256), 256, 0, st>>>(nrows, s, rp, col, val, X, Y); count_launch(); }
-}
-
-// z = (FP64) Xsub[owning copy] + (FP64) q  (prolongation of the FP32 local solutions)
-__global__ void k_scatter_owned_fq(const int* __restrict__ own, int64_t n, const float2* __restrict__ Xsub,
-                                   const float2* __restrict__ Q, double2* __restrict__ Z, int s) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  if (r >= n) return;
-  const float2 v = Xsub[(int64_t)own[r] * s + (g - r * s)];
-  const float2 q = Q[g];
-  Z[g] = make_double2((double)v.x + (double)q.x, (double)v.y + (double)q.y);
-}
-void scatter_owned_fq(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
-                      cudaStream_t st) {
-  if (n * s) { k_scatter_owned_fq<<<grid_for(n * s, 256), 256, 0, st>>>(own, n, Xsub, Q, Z, s); count_launch(); }
-}
-
-__global__ void k_gather_ff(const int* __restrict__ idx, int64_t nrows, const float2* __restrict__ X,
-                            float2* __restrict__ Y, int s) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  if (r >= nrows) return;
-  Y[g] = X[(int64_t)idx[r] * s + (g - r * s)];
-}
-void gather_rows_ff(const int* idx, int64_t nrows, const float2* X, float2* Y, int s, cudaStream_t st) {
-  if (nrows * s) { k_gather_ff<<<grid_for(nrows * s, 256), 256, 0, st>>>(idx, nrows, X, Y, s); count_launch(); }
-}
-
-__global__ void k_scatter_ff(const int* __restrict__ own, int64_t n, const float2* __restrict__ Xsub,
-                             float2* __restrict__ Z, int s) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  if (r >= n) return;
-  Z[g] = Xsub[(int64_t)own[r] * s + (g - r * s)];
-}
-void scatter_owned_ff(const int* own, int64_t n, const float2* Xsub, float2* Z, int s, cudaStream_t st) {
-  if (n * s) { k_scatter_ff<<<grid_for(n * s, 256), 256, 0, st>>>(own, n, Xsub, Z, s); count_launch(); }
 }
 
 __global__ void k_d2f(const double2* __restrict__ X, float2* __restrict__ Y, int64_t count) {
