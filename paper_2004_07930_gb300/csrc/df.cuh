@@ -41,6 +41,29 @@ static __device__ __forceinline__ double f2d(float f) {
       (long long)(sign | ((unsigned long long)(e - 127 + 1023) << 52) | ((unsigned long long)(u & 0x7FFFFFu) << 29)));
 }
 
+// hi + lo as FP64 for a renormalised pair (|lo| <= ulp(hi)), by integer
+// instructions: hi's significand moved up by 29 bits plus lo in units of its
+// last place, rounded to nearest: the same bits as the FP64 sum. Pairs whose
+// sum falls below hi's power of two, others, and values outside the range in
+// which the units are normal FP32 numbers, go through the FP64 pipe.
+static __device__ __forceinline__ double df_join(float hi, float lo) {
+  const unsigned u = __float_as_uint(hi);
+  const int e = (int)((u >> 23) & 0xFFu);  // hi = 1.f 2^(e - 127)
+  if (e < 60 || e > 190 || fabsf(lo) > __uint_as_float((unsigned)(e - 23) << 23)) return f2d(hi) + f2d(lo);
+  // one unit = 2^(e - 127 - 52); lo in units, |lo| <= 2^29
+  const int l = __float2int_rn(__fmul_rn(lo, __uint_as_float((unsigned)(306 - e) << 23)));
+  long long m = ((long long)((u & 0x7FFFFFu) | 0x800000u)) << 29;
+  m += (u >> 31) ? -(long long)l : (long long)l;
+  long long ex = e - 127 + 1023;
+  if (m < (1ll << 52)) return f2d(hi) + f2d(lo);  // one more bit would be needed
+  if (m >= (1ll << 53)) {                         // the next power of two itself
+    m >>= 1;
+    ++ex;
+  }
+  return __longlong_as_double((long long)((unsigned long long)(u & 0x80000000u) << 32) | (ex << 52) |
+                              (m & 0xFFFFFFFFFFFFFll));
+}
+
 // (sh, sl) += (ah + al) (xh + xl); the al*xl term (2^-48 relative) is dropped
 static __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al, float xh, float xl) {
   const float p = __fmul_rn(ah, xh);

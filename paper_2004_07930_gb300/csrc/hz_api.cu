@@ -783,7 +783,7 @@ struct hz_ctx {
 
 namespace {
 
-void alloc_krylov(DevKrylov& K, int64_t n, int s, int m, DevPool& p, bool fp32, bool df = false) {
+void alloc_krylov(DevKrylov& K, int64_t n, int s, int m, DevPool& p, cudaStream_t st, bool fp32, bool df = false) {
   K.n = n;
   K.s = s;
   K.m = m;
@@ -799,7 +799,7 @@ void alloc_krylov(DevKrylov& K, int64_t n, int s, int m, DevPool& p, bool fp32, 
   K.Zk = p.alloc<char>((size_t)m * n * s * es);
   K.W = p.alloc<char>((size_t)n * s * es);
   K.H = p.alloc<double2>((size_t)s * (m + 1) * m);
-  K.hpart = p.alloc<double2>((size_t)K.nblk * (m + 1) * s);
+  K.hpart = p.alloc<double2>((size_t)K.nblk * (m + 2) * s);
   K.h1 = p.alloc<double2>((size_t)(m + 1) * s);
   K.h2 = p.alloc<double2>((size_t)(m + 1) * s);
   K.cs = p.alloc<double>((size_t)s * m);
@@ -812,6 +812,8 @@ void alloc_krylov(DevKrylov& K, int64_t n, int s, int m, DevPool& p, bool fp32, 
   K.kc = p.alloc<int>(s);
   K.done = p.alloc<int>(s);
   K.reorth = p.alloc<int>(s);
+  K.count = p.alloc<int>(s);
+  CK(cudaMemsetAsync(K.count, 0, s * sizeof(int), st));
 }
 
 void ensure_workspace(hz_ctx* c, int s) {
@@ -844,7 +846,7 @@ void ensure_workspace(hz_ctx* c, int s) {
   if (c->lf.mf.tc) c->lf.mf.P = p.alloc<char>((size_t)c->lf.mf.max_slots * MF_TILE_ROWS * cols * ef);
   c->lf.mf.s_cap = s;
   // double-float Arnoldi for the outer space unless block FGMRES or recycling (which read W in FP64)
-  alloc_krylov(c->Kout, n, s, c->opt.restart, p, false,
+  alloc_krylov(c->Kout, n, s, c->opt.restart, p, c->st, false,
                c->df && !c->opt.block_arnoldi && c->opt.recycle == 0);
   if (c->df) {
     c->Xdf = p.alloc<float4>(n * s);
@@ -894,7 +896,7 @@ void ensure_workspace(hz_ctx* c, int s) {
     if (c->lc.mf.tc) c->lc.mf.P = p.alloc<char>((size_t)c->lc.mf.max_slots * MF_TILE_ROWS * cols * ec);
     c->lc.mf.s_cap = s;
     if (c->opt.coarse_mode == HZ_COARSE_GMRES) {
-      alloc_krylov(c->Kin, nh, s, std::max(1, c->opt.coarse_inner_its), p, c->coarse32, c->df);
+      alloc_krylov(c->Kin, nh, s, std::max(1, c->opt.coarse_inner_its), p, c->st, c->coarse32, c->df);
       CK(cudaMemsetAsync(c->Kin.tol, 0, s * sizeof(double), c->st));
     }
     if (c->coarse32) {

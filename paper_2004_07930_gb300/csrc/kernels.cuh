@@ -254,7 +254,7 @@ struct DevKrylov {
   void* Zk = nullptr;       // [m][n][s]
   void* W = nullptr;        // [n][s]
   double2* H = nullptr;     // [s][(m+1) m] Hessenberg, rotated in place
-  double2* hpart = nullptr; // partial dot products [nblk][m+1][s]
+  double2* hpart = nullptr; // partial dot products [nblk][m+2][s]
   double2* h1 = nullptr;    // [m+1][s]
   double2* h2 = nullptr;    // [m+1][s]
   double* cs = nullptr;     // [s][m] Givens cosines (real)
@@ -267,6 +267,7 @@ struct DevKrylov {
   int* kc = nullptr;        // [s] accepted Arnoldi steps
   int* done = nullptr;      // [s]
   int* reorth = nullptr;    // [s] second Gram-Schmidt pass needed
+  int* count = nullptr;     // [s] finished CTAs of a sum (zero between launches)
   double2* Hraw = nullptr;  // [s][(m+1) m] unrotated Hessenberg (recycling only; may be NULL)
   int nblk = 0;
   // double-float Arnoldi (FP64 Krylov spaces of the mixed form, emulate_fp64): A z arrives in
