@@ -23,6 +23,7 @@
 
 #include "df.cuh"
 #include "kernels.cuh"
+#include "spmm.cuh"
 
 namespace hz {
 
@@ -38,84 +39,67 @@ __global__ void k_to_df(const double2* __restrict__ X, float4* __restrict__ Y, i
   Y[g] = make_float4(r.x, r.y, i.x, i.y);
 }
 
-// Y = (A_re + i A_im) X or Y = B - A X, X in double-float; one thread per
-// (row, column), the s threads of a row share the index and value loads.
-// With Ydf the product A X is written in double-float instead (renormalised).
-__global__ void k_spmm_df(int64_t n, int s, const int64_t* __restrict__ rp_re, const int32_t* __restrict__ col_re,
-                          const float2* __restrict__ val_re, const int64_t* __restrict__ rp_im,
-                          const int32_t* __restrict__ col_im, const float2* __restrict__ val_im,
-                          const float4* __restrict__ X, double2* __restrict__ Y, const double2* __restrict__ B,
-                          int mode, float4* __restrict__ Ydf) {
-  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t r = g / s;
-  const int c = (int)(g - r * s);
-  if (r >= n) return;
-  float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-#pragma unroll 4
-  for (int64_t p = rp_re[r], pe = rp_re[r + 1]; p < pe; ++p) {
-    const float2 a = val_re[p];
-    const float4 x = X[(int64_t)col_re[p] * s + c];
-    df_mac(rh, rl, a.x, a.y, x.x, x.y);
-    df_mac(ih, il, a.x, a.y, x.z, x.w);
+namespace {
+struct OutRows {  // Y = A X, or B - A X
+  double2* Y;
+  const double2* B;
+  int s;
+  __device__ __forceinline__ void operator()(int64_t r, int c, float4 a) const {
+    const int64_t g = r * s + c;
+    const double2 y = SpDf<float4>::to_d(a);
+    if (B) {
+      const double2 b = B[g];
+      Y[g] = make_double2(b.x - y.x, b.y - y.y);
+    } else {
+      Y[g] = y;
+    }
   }
-#pragma unroll 4
-  for (int64_t p = rp_im[r], pe = rp_im[r + 1]; p < pe; ++p) {
-    const float2 b = val_im[p];
-    const float4 x = X[(int64_t)col_im[p] * s + c];
-    df_mac(rh, rl, -b.x, -b.y, x.z, x.w);  // re -= b im(x)
-    df_mac(ih, il, b.x, b.y, x.x, x.y);    // im += b re(x)
+};
+struct OutCols {  // Y = A X with the columns contiguous, [s][n]
+  double2* Y;
+  int64_t n;
+  __device__ __forceinline__ void operator()(int64_t r, int c, float4 a) const {
+    Y[(int64_t)c * n + r] = SpDf<float4>::to_d(a);
   }
-  if (Ydf) {
-    df_norm(rh, rl);
-    df_norm(ih, il);
-    Ydf[g] = make_float4(rh, rl, ih, il);
-    return;
+};
+struct OutDf {  // Y = A X in double-float, renormalised
+  float4* Y;
+  int s;
+  __device__ __forceinline__ void operator()(int64_t r, int c, float4 a) const {
+    df_norm(a.x, a.y);
+    df_norm(a.z, a.w);
+    Y[r * s + c] = a;
   }
-  const double ar = f2d(rh) + f2d(rl), ai = f2d(ih) + f2d(il);
-  if (mode == 1) {
-    const double2 b = B[g];
-    Y[g] = make_double2(b.x - ar, b.y - ai);
-  } else {
-    Y[g] = make_double2(ar, ai);
-  }
+};
+template <typename XT, typename Out>
+void spmm_df(const DevSplitCsr& A, const XT* X, Out out, int s, cudaStream_t st, bool ordered = false) {
+  spmm_launch<SpDf<XT>>(A.n, s, A.rp_re, A.col_re, A.val_re_df, A.rp_im, A.col_im, A.val_im_df, X, out, st, ordered);
 }
-
-// Y = R X for a real CSR R (the coarse restriction Z^T and prolongation Z),
-// X in double-float, Y in FP64
-__global__ void k_spmm_real_df(int64_t n, int s, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                               const float2* __restrict__ val, const float4* __restrict__ X, double2* __restrict__ Y) {
-  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t r = g / s;
-  const int c = (int)(g - r * s);
-  if (r >= n) return;
-  float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-#pragma unroll 4
-  for (int64_t p = rp[r], pe = rp[r + 1]; p < pe; ++p) {
-    const float2 a = val[p];
-    const float4 x = X[(int64_t)col[p] * s + c];
-    df_mac(rh, rl, a.x, a.y, x.x, x.y);
-    df_mac(ih, il, a.x, a.y, x.z, x.w);
-  }
-  Y[g] = make_double2(f2d(rh) + f2d(rl), f2d(ih) + f2d(il));
-}
+}  // namespace
 
 void spmm_real_df(int64_t nrows, const int64_t* rp, const int32_t* col, const float2* val, const float4* X,
                   double2* Y, int s, cudaStream_t st) {
-  const int64_t work = nrows * s;
-  if (work == 0) return;
-  { k_spmm_real_df<<<grid_for(work, 256), 256, 0, st>>>(nrows, s, rp, col, val, X, Y); count_launch(); }
+  spmm_launch<SpDf<float4>>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRows{Y, nullptr, s}, st, true);
 }
 
 void to_df(const double2* X, float4* Y, int64_t count, cudaStream_t st) {
   if (count) { k_to_df<<<grid_for(count, 256), 256, 0, st>>>(X, Y, count); count_launch(); }
 }
 
-void spmm_split_df(const DevSplitCsr& A, const float4* X, double2* Y, const double2* B, int s, int mode,
-                   cudaStream_t st, float4* Ydf) {
-  const int64_t work = A.n * s;
-  if (work == 0) return;
-  { k_spmm_df<<<grid_for(work, 256), 256, 0, st>>>(A.n, s, A.rp_re, A.col_re, A.val_re_df, A.rp_im, A.col_im,
-                                                  A.val_im_df, X, Y, B, mode, Ydf); count_launch(); }
+void spmm_split_df(const DevSplitCsr& A, const float4* X, double2* Y, const double2* B, int s, cudaStream_t st) {
+  spmm_df(A, X, OutRows{Y, B, s}, s, st, B != nullptr);  // t = v - A q feeds FP32 local solves: in storage order
+}
+void spmm_split_df_cols(const DevSplitCsr& A, const float4* X, double2* Y, int s, cudaStream_t st) {
+  spmm_df(A, X, OutCols{Y, A.n}, s, st);
+}
+void spmm_split_df(const DevSplitCsr& A, const float4* X, float4* Y, int s, cudaStream_t st) {
+  spmm_df(A, X, OutDf{Y, s}, s, st);
+}
+void spmm_split_df(const DevSplitCsr& A, const float2* X, double2* Y, int s, cudaStream_t st) {
+  spmm_df(A, X, OutRows{Y, nullptr, s}, s, st);
+}
+void spmm_split_df(const DevSplitCsr& A, const float2* X, float4* Y, int s, cudaStream_t st, bool ordered) {
+  spmm_df(A, X, OutDf{Y, s}, s, st, ordered);
 }
 
 }  // namespace hz

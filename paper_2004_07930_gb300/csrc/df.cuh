@@ -77,6 +77,27 @@ static __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, fl
   sh = t;
 }
 
+// the same with xl = 0
+static __device__ __forceinline__ void df_mac_f(float& sh, float& sl, float ah, float al, float xh) {
+  const float p = __fmul_rn(ah, xh);
+  float e = __fmaf_rn(ah, xh, -p);
+  e = __fmaf_rn(al, xh, e);
+  const float t = __fadd_rn(sh, p);
+  const float z = __fsub_rn(t, sh);
+  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, z)), __fsub_rn(p, z));
+  sl = __fadd_rn(sl, __fadd_rn(err, e));
+  sh = t;
+}
+
+// (sh, sl) += (h, l)
+static __device__ __forceinline__ void df_add(float& sh, float& sl, float h, float l) {
+  const float t = __fadd_rn(sh, h);
+  const float z = __fsub_rn(t, sh);
+  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, z)), __fsub_rn(h, z));
+  sl = __fadd_rn(sl, __fadd_rn(err, l));
+  sh = t;
+}
+
 // renormalise (h, l) so that |l| is at most half an ulp of h (Fast2Sum; |h| >= |l| or h = 0)
 static __device__ __forceinline__ void df_norm(float& h, float& l) {
   const float t = __fadd_rn(h, l);

@@ -738,7 +738,9 @@ struct hz_ctx {
   bool has_coarse = false;
   bool coarse32 = false;      // mixed form with coarse_fp32: the whole of M^{-1} on FP32 blocks
   bool df = false;            // mixed form with emulate_fp64: products with A and E in double-float
-  float4 *Xdf = nullptr, *XdfH = nullptr;  // double-float copies of the product's input block (fine, coarse)
+  // operands of the double-float products (fine, coarse): the input block in double-float, and in FP32
+  float4 *Xdf = nullptr, *XdfH = nullptr;
+  float2 *Xf = nullptr, *XfH = nullptr;
   Space cspace;
   DevSplitCsr E;
   DevReal Z, ZT;
@@ -850,7 +852,11 @@ void ensure_workspace(hz_ctx* c, int s) {
                c->df && !c->opt.block_arnoldi && c->opt.recycle == 0);
   if (c->df) {
     c->Xdf = p.alloc<float4>(n * s);
-    if (c->has_coarse && !c->coarse32) c->XdfH = p.alloc<float4>(c->cspace.n * s);
+    if (!c->has_coarse) c->Xf = reinterpret_cast<float2*>(c->Xdf);  // one or the other is in use
+    if (c->has_coarse && !c->coarse32) {
+      c->XdfH = p.alloc<float4>(c->cspace.n * s);
+      c->XfH = reinterpret_cast<float2*>(c->XdfH);
+    }
   }
   if (c->opt.recycle > 0) {
     const int rk = c->opt.recycle, m = c->opt.restart;
@@ -940,8 +946,9 @@ void run_graph(GraphCache* g, int s, cudaStream_t st, F&& body) {
 }
 
 // ORAS on one level: Z = sum_i R_i^T D_i A_i^{-1} R_i V (+ Qadd)
+// (Zdf, Zf: the operand of the product that follows, see scatter_owned)
 void apply_oras(LevelDev& L, const double2* V, double2* Zout, const double2* Qadd, double2* Xsub, int s,
-                cudaStream_t st, Profiler* prof = nullptr, GraphCache* graph = nullptr) {
+                cudaStream_t st, float4* Zdf, float2* Zf, Profiler* prof = nullptr, GraphCache* graph = nullptr) {
   const double es = L.mf.fp32 ? 8.0 : 16.0;
   // gather: indices + read V rows + write sub-vector; scatter: owner index + read + (q) + write
   const double rbytes = 4.0 * L.sub_rows + (16.0 + es) * L.sub_rows * s + 4.0 * L.n +
@@ -959,7 +966,7 @@ void apply_oras(LevelDev& L, const double2* V, double2* Zout, const double2* Qad
   if (prof) prof->end(p1, st, fflops, fbytes);
   int p2 = prof ? prof->begin(PH_RESTRICT, st) : -1;
   if (L.mf.fp32)
-    scatter_owned(L.mf.own, L.n, (const float2*)Xsub, Qadd, Zout, s, st);
+    scatter_owned(L.mf.own, L.n, (const float2*)Xsub, Qadd, Zout, s, st, Zdf, Zf);
   else
     scatter_owned(L.mf.own, L.n, Xsub, Qadd, Zout, s, st);
   if (prof) prof->end(p2, st, 0.0, rbytes);
@@ -973,7 +980,7 @@ void coarse_solve(hz_ctx* c, const double2* rH, double2* yH, int s) {
   const int64_t nh = c->cspace.n;
   LevelDev& L = c->lc;
   if (c->opt.coarse_mode == HZ_COARSE_DIRECT) {
-    apply_oras(L, rH, yH, nullptr, c->XsubH, s, st);
+    apply_oras(L, rH, yH, nullptr, c->XsubH, s, st, nullptr, nullptr);
     return;
   }
   DevKrylov& K = c->Kin;
@@ -1002,13 +1009,11 @@ void coarse_solve(hz_ctx* c, const double2* rH, double2* yH, int s) {
   axpy_cols_zero(yH, vs, st);
   krylov_start(K, rH, st);
   for (int j = 0; j < K.m; ++j) {
-    apply_oras(L, V + j * vs, Zk + j * vs, nullptr, c->XsubH, s, st);
-    if (c->df) {
-      to_df(Zk + j * vs, c->XdfH, vs, st);
-      spmm_split_df(c->E, c->XdfH, (double2*)K.W, nullptr, s, 0, st, K.df ? K.Wdf : nullptr);
-    } else {
-      spmm_split(c->E, Zk + j * vs, (double2*)K.W, nullptr, s, 0, st);
-    }
+    apply_oras(L, V + j * vs, Zk + j * vs, nullptr, c->XsubH, s, st, nullptr, c->df ? c->XfH : nullptr);
+    if (c->df)  // coarse ORAS has FP32 values: E times them in FP32 operands
+      spmm_split_df(c->E, c->XfH, K.Wdf, s, st, true);
+    else
+      spmm_split(c->E, Zk + j * vs, (double2*)K.W, nullptr, s, st, true);
     krylov_arnoldi(K, j, st);
   }
   krylov_update(K, yH, st);
@@ -1021,26 +1026,39 @@ static void spmm_cost(const DevSplitCsr& A, int s, bool with_b, double& flops, d
   bytes = 12.0 * nz + 16.0 * (A.n + 1) + 16.0 * A.ncols * s + 16.0 * A.n * s * (with_b ? 2.0 : 1.0);
 }
 
-void spmm_A(hz_ctx* c, const double2* X, double2* Y, const double2* B, int s, int mode) {
+// Y = A X, or B - A X when B is given
+void spmm_A(hz_ctx* c, const double2* X, double2* Y, const double2* B, int s) {
   double fl, by;
-  spmm_cost(c->A, s, mode == 1, fl, by);
+  spmm_cost(c->A, s, B != nullptr, fl, by);
   int id = c->prof.begin(PH_SPMM, c->st);
   if (c->df) {
     to_df(X, c->Xdf, c->space.n * s, c->st);
-    spmm_split_df(c->A, c->Xdf, Y, B, s, mode, c->st);
+    spmm_split_df(c->A, c->Xdf, Y, B, s, c->st);
   } else {
-    spmm_split(c->A, X, Y, B, s, mode, c->st);
+    spmm_split(c->A, X, Y, B, s, c->st);
   }
   c->prof.end(id, c->st, fl, by);
 }
 
-// A X into a double-float block (the Krylov product of the double-float Arnoldi)
-void spmm_A_df(hz_ctx* c, const double2* X, float4* Ydf, int s) {
+// The Krylov product w = A z of the mixed form with emulate_fp64, z as the
+// preconditioner's scatter left it: in FP32 (c->Xf) when the coarse level adds
+// nothing to it, else in double-float (c->Xdf). Wdf: double-float w for the
+// double-float Arnoldi, else FP64 W.
+void spmm_A_z(hz_ctx* c, double2* W, float4* Wdf, int s) {
   double fl, by;
   spmm_cost(c->A, s, false, fl, by);
   int id = c->prof.begin(PH_SPMM, c->st);
-  to_df(X, c->Xdf, c->space.n * s, c->st);
-  spmm_split_df(c->A, c->Xdf, nullptr, nullptr, s, 0, c->st, Ydf);
+  if (!c->has_coarse) {
+    if (Wdf)
+      spmm_split_df(c->A, c->Xf, Wdf, s, c->st);
+    else
+      spmm_split_df(c->A, c->Xf, W, s, c->st);
+  } else {
+    if (Wdf)
+      spmm_split_df(c->A, c->Xdf, Wdf, s, c->st);
+    else
+      spmm_split_df(c->A, c->Xdf, W, nullptr, s, c->st);
+  }
   c->prof.end(id, c->st, fl, by);
 }
 
@@ -1085,7 +1103,7 @@ void apply_prec(hz_ctx* c, const double2* V, double2* Zout, int s) {
   cudaStream_t st = c->st;
   GraphCache* gf = c->opt.use_graphs ? &c->g_fronts : nullptr;
   if (!c->has_coarse) {
-    apply_oras(c->lf, V, Zout, nullptr, c->Xsub, s, st, &c->prof, gf);
+    apply_oras(c->lf, V, Zout, nullptr, c->Xsub, s, st, nullptr, c->df ? c->Xf : nullptr, &c->prof, gf);
     return;
   }
   if (c->lf.mf.fp32 && c->v32 && c->opt.coarse_mode == HZ_COARSE_GMRES) {
@@ -1115,7 +1133,7 @@ void apply_prec(hz_ctx* c, const double2* V, double2* Zout, int s) {
     c->prof.end(p1, st, 8.0 * s * 2.0 * L.info.factor_entries,
                 8.0 * 2.0 * L.info.factor_entries + 2.0 * 8.0 * s * L.sub_rows);
     int p2 = c->prof.begin(PH_RESTRICT, st);
-    scatter_owned(L.mf.own, L.n, (const float2*)c->Xsub, c->q32, Zout, s, st);     // z = M1^{-1} t + q
+    scatter_owned(L.mf.own, L.n, (const float2*)c->Xsub, c->q32, Zout, s, st, c->df ? c->Xdf : nullptr);  // z = M1^{-1} t + q
     c->prof.end(p2, st, 0.0, 4.0 * L.sub_rows + 16.0 * L.sub_rows * s + 4.0 * L.n + 32.0 * L.n * s);
     return;
   }
@@ -1139,8 +1157,8 @@ void apply_prec(hz_ctx* c, const double2* V, double2* Zout, int s) {
     coarse_cost(c, s, false, cf, cb);
     c->prof.end(id, st, cf, cb);
   }
-  spmm_A(c, c->Q, c->T, V, s, 1);                                         // t = v - A q
-  apply_oras(c->lf, c->T, Zout, c->Q, c->Xsub, s, st, &c->prof, gf);      // z = M1^{-1} t + q
+  spmm_A(c, c->Q, c->T, V, s);                                         // t = v - A q
+  apply_oras(c->lf, c->T, Zout, c->Q, c->Xsub, s, st, c->df ? c->Xdf : nullptr, nullptr, &c->prof, gf);      // z = M1^{-1} t + q
 }
 
 // One restart cycle of flexible GMRES on the block: Krylov space from the
@@ -1161,10 +1179,10 @@ int fgmres_cycle(hz_ctx* c, int s, int max_its, bool recyc = false) {
   int its = 0;
   for (int j = 0; j < m; ++j) {
     apply_prec(c, (double2*)K.V + j * vs, (double2*)K.Zk + j * vs, s);
-    if (K.df)
-      spmm_A_df(c, (double2*)K.Zk + j * vs, K.Wdf, s);
+    if (c->df)
+      spmm_A_z(c, (double2*)K.W, K.df ? K.Wdf : nullptr, s);
     else
-      spmm_A(c, (double2*)K.Zk + j * vs, (double2*)K.W, nullptr, s, 0);
+      spmm_A(c, (double2*)K.Zk + j * vs, (double2*)K.W, nullptr, s);
     int id = c->prof.begin(PH_ARNOLDI, st);
     if (rk > 0) {  // B_j = C^H w, w -= C B_j
       double2* Bj = c->Bc + (size_t)j * rk * s;
@@ -1250,7 +1268,7 @@ void recycle_update(hz_ctx* c, int s, const std::vector<int>& kc) {
   const int total = std::min(RK, c->rk_eff + knew), kold = total - knew;
   // new directions and their images: Rt1 = Z P, Rt2 = A Rt1 ([n][knew])
   recycle_build((const double2*)c->Kout.Zk, n * s, s, col, c->Rp, me, knew, c->Rt1, knew, 0, n, st);
-  spmm_split(c->A, c->Rt1, c->Rt2, nullptr, knew, 0, st);
+  spmm_split(c->A, c->Rt1, c->Rt2, nullptr, knew, st);
   recycle_copy(c->Rt1, knew, 0, c->Un, total, 0, knew, n, st);
   recycle_copy(c->Rt2, knew, 0, c->Cn, total, 0, knew, n, st);
   if (kold > 0) {
@@ -1289,7 +1307,7 @@ int fgmres_cycle_block(hz_ctx* c, int s, int max_its) {
   int its = 0;
   for (int j = 0; j < m; ++j) {
     apply_prec(c, B.V + j * vs, B.Zk + j * vs, s);
-    spmm_A(c, B.Zk + j * vs, B.W, nullptr, s, 0);
+    spmm_A(c, B.Zk + j * vs, B.W, nullptr, s);
     int id = c->prof.begin(PH_ARNOLDI, st);
     block_krylov_arnoldi(B, j, st);
     // two CGS passes (Gram blocks + update) over V_0..j, then CholQR2 (two Gram + triangular solves)
@@ -1309,7 +1327,7 @@ int fgmres_cycle_block(hz_ctx* c, int s, int max_its) {
 void true_residual(hz_ctx* c, int s) {
   cudaStream_t st = c->st;
   const int64_t n = c->space.n;
-  spmm_A(c, c->X, c->R, c->B, s, 1);
+  spmm_A(c, c->X, c->R, c->B, s);
   column_norms(c->R, n, s, c->rnorm, c->Kout, st);
   CK(cudaMemcpyAsync(c->h_res, c->rnorm, s * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -1814,15 +1832,43 @@ static void store_block(hz_ctx* c, const double2* Brow, double* out, int s, int 
   CK(cudaStreamSynchronize(c->st));
 }
 
+// Y = A X: the input goes straight to the product's operand (double-float in
+// the mixed form with emulate_fp64) and the product writes [s][n], so that
+// neither side has an FP64 [n][s] block in between. One column on the device
+// needs no operand of its own unless the caller's buffers overlap.
 int hz_apply_A(hz_ctx* c, const double* X, double* Y, int32_t s, int32_t on_device) {
   if (!c || !X || !Y || s < 1 || s > c->opt.max_block) return fail(HZ_EINVAL, "bad argument");
   return guarded([&]() -> int {
     join_user(c);
     ensure_workspace(c, s);
-    load_block(c, X, s, on_device);
-    spmm_A(c, c->B, c->R, nullptr, s, 0);  // recorded in the "spmm_A" phase while profiling
+    const int64_t n = c->space.n;
+    const size_t bytes = (size_t)n * s * sizeof(double2);
+    const double2* src = reinterpret_cast<const double2*>(X);
+    double2* dst = on_device ? reinterpret_cast<double2*>(Y) : c->R;
+    if (!on_device) {
+      CK(cudaMemcpyAsync(c->U, X, bytes, cudaMemcpyHostToDevice, c->st));
+      src = c->U;
+    }
+    double fl, by;
+    spmm_cost(c->A, s, false, fl, by);
+    if (c->df) {
+      transpose_to_rows(src, c->Xdf, n, s, c->st);
+      const int id = c->prof.begin(PH_SPMM, c->st);
+      spmm_split_df_cols(c->A, c->Xdf, dst, s, c->st);
+      c->prof.end(id, c->st, fl, by);
+    } else {
+      const uintptr_t a = (uintptr_t)src, b = (uintptr_t)dst;
+      if (s > 1 || (a < b ? b - a : a - b) < bytes) {
+        transpose_to_rows(src, c->B, n, s, c->st);
+        src = c->B;
+      }
+      const int id = c->prof.begin(PH_SPMM, c->st);
+      spmm_split_cols(c->A, src, dst, s, c->st);
+      c->prof.end(id, c->st, fl, by);
+    }
     check_launch();
-    store_block(c, c->R, Y, s, on_device);
+    if (!on_device) CK(cudaMemcpyAsync(Y, dst, bytes, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
     return HZ_OK;
   });
 }

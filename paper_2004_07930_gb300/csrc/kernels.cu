@@ -14,6 +14,7 @@
 #include <cstdio>
 
 #include "kernels.cuh"
+#include "spmm.cuh"
 
 namespace hz {
 
@@ -42,72 +43,40 @@ __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.
 static inline unsigned grid_for(int64_t work, int block) { return (unsigned)((work + block - 1) / block); }
 
 // ---------------------------------------------------------------------------
-// SpMM: Y = (A_re + i A_im) X  or  Y = B - A X   (K1)
-// one thread per (row, column); the s threads of a row share the index and
-// value loads, the X loads of one nonzero are one contiguous 16 s-byte row.
+// SpMM: Y = (A_re + i A_im) X  or  Y = B - A X   (K1), native FP64
 // ---------------------------------------------------------------------------
-__global__ void k_spmm_split(int64_t n, int s, const int64_t* __restrict__ rp_re, const int32_t* __restrict__ col_re,
-                             const double* __restrict__ val_re, const int64_t* __restrict__ rp_im,
-                             const int32_t* __restrict__ col_im, const double* __restrict__ val_im,
-                             const double2* __restrict__ X, double2* __restrict__ Y, const double2* __restrict__ B,
-                             int mode) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  int c = (int)(g - r * s);
-  if (r >= n) return;
-  double ar = 0.0, ai = 0.0;
-  #pragma unroll 4
-  for (int64_t p = rp_re[r], pe = rp_re[r + 1]; p < pe; ++p) {
-    double a = val_re[p];
-    double2 x = X[(int64_t)col_re[p] * s + c];
-    ar = fma(a, x.x, ar);
-    ai = fma(a, x.y, ai);
+namespace {
+struct OutRows {
+  double2* Y;
+  const double2* B;
+  int s;
+  __device__ __forceinline__ void operator()(int64_t r, int c, double2 y) const {
+    const int64_t g = r * s + c;
+    if (B) {
+      const double2 b = B[g];
+      y = make_double2(b.x - y.x, b.y - y.y);
+    }
+    Y[g] = y;
   }
-  #pragma unroll 4
-  for (int64_t p = rp_im[r], pe = rp_im[r + 1]; p < pe; ++p) {
-    double b = val_im[p];
-    double2 x = X[(int64_t)col_im[p] * s + c];
-    ar = fma(-b, x.y, ar);
-    ai = fma(b, x.x, ai);
-  }
-  if (mode == 1) {
-    double2 b = B[g];
-    Y[g] = make_double2(b.x - ar, b.y - ai);
-  } else {
-    Y[g] = make_double2(ar, ai);
-  }
-}
+};
+struct OutCols {  // Y = A X with the columns contiguous, [s][n]
+  double2* Y;
+  int64_t n;
+  __device__ __forceinline__ void operator()(int64_t r, int c, double2 y) const { Y[(int64_t)c * n + r] = y; }
+};
+}  // namespace
 
-void spmm_split(const DevSplitCsr& A, const double2* X, double2* Y, const double2* B, int s, int mode,
-                cudaStream_t st) {
-  int64_t work = A.n * s;
-  if (work == 0) return;
-  { k_spmm_split<<<grid_for(work, 256), 256, 0, st>>>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im,
-                                                    A.val_im, X, Y, B, mode); count_launch(); }
+void spmm_split(const DevSplitCsr& A, const double2* X, double2* Y, const double2* B, int s, cudaStream_t st,
+                bool ordered) {
+  spmm_launch<SpF64>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im, A.val_im, X, OutRows{Y, B, s}, st, ordered);
 }
-
-__global__ void k_spmm_real(int64_t n, int s, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                            const double* __restrict__ val, const double2* __restrict__ X, double2* __restrict__ Y) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  int c = (int)(g - r * s);
-  if (r >= n) return;
-  double ar = 0.0, ai = 0.0;
-  #pragma unroll 4
-  for (int64_t p = rp[r], pe = rp[r + 1]; p < pe; ++p) {
-    double a = val[p];
-    double2 x = X[(int64_t)col[p] * s + c];
-    ar = fma(a, x.x, ar);
-    ai = fma(a, x.y, ai);
-  }
-  Y[g] = make_double2(ar, ai);
+void spmm_split_cols(const DevSplitCsr& A, const double2* X, double2* Y, int s, cudaStream_t st) {
+  spmm_launch<SpF64>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im, A.val_im, X, OutCols{Y, A.n}, st);
 }
 
 void spmm_real(int64_t nrows, const int64_t* rp, const int32_t* col, const double* val, const double2* X,
                double2* Y, int s, cudaStream_t st) {
-  int64_t work = nrows * s;
-  if (work == 0) return;
-  { k_spmm_real<<<grid_for(work, 256), 256, 0, st>>>(nrows, s, rp, col, val, X, Y); count_launch(); }
+  spmm_launch<SpF64>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRows{Y, nullptr, s}, st, true);
 }
 
 // ---------------------------------------------------------------------------
@@ -132,9 +101,16 @@ __global__ void k_gather(const int* __restrict__ idx, int64_t nrows, const In* _
   Y[r * cols + c] = y;
 }
 
+// the operand of the product that follows: z in double-float, or in FP32 where z has no more
+__device__ __forceinline__ void put_copy(float4* p, double2 z) {
+  const float2 a = df_split(z.x), b = df_split(z.y);
+  *p = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void put_copy(float4* p, float2 z) { *p = make_float4(z.x, 0.f, z.y, 0.f); }
+
 template <typename In, typename Q, typename Out>
 __global__ void k_scatter(const int* __restrict__ own, int64_t n, const In* __restrict__ Xsub, const Q* __restrict__ Qb,
-                          Out* __restrict__ Z, int s, int cols) {
+                          Out* __restrict__ Z, int s, int cols, float4* __restrict__ Zdf, float2* __restrict__ Zf) {
   const int64_t r = blockIdx.x * (int64_t)blockDim.y + threadIdx.y;
   const int c = threadIdx.x;
   if (r >= n) return;
@@ -148,6 +124,8 @@ __global__ void k_scatter(const int* __restrict__ own, int64_t n, const In* __re
     z.y += (decltype(z.y))q.y;
   }
   Z[r * s + c] = z;
+  if (Zdf) put_copy(Zdf + r * s + c, z);
+  if (Zf) Zf[r * s + c] = make_float2((float)x.x, (float)x.y);
 }
 
 template <typename In, typename Out>
@@ -158,10 +136,11 @@ static void gather_t(const int* idx, int64_t nrows, const In* X, Out* Y, int s, 
   { k_gather<<<grid_for(nrows, b.y), b, 0, st>>>(idx, nrows, X, Y, s, cols); count_launch(); }
 }
 template <typename In, typename Q, typename Out>
-static void scatter_t(const int* own, int64_t n, const In* Xsub, const Q* Qb, Out* Z, int s, cudaStream_t st) {
+static void scatter_t(const int* own, int64_t n, const In* Xsub, const Q* Qb, Out* Z, int s, cudaStream_t st,
+                      float4* Zdf = nullptr, float2* Zf = nullptr) {
   if (n * s == 0) return;
   const dim3 b(s, std::max(1, 256 / s));
-  { k_scatter<<<grid_for(n, b.y), b, 0, st>>>(own, n, Xsub, Qb, Z, s, sweep_cols(s)); count_launch(); }
+  { k_scatter<<<grid_for(n, b.y), b, 0, st>>>(own, n, Xsub, Qb, Z, s, sweep_cols(s), Zdf, Zf); count_launch(); }
 }
 
 void gather_rows(const int* idx, int64_t nrows, const double2* X, double2* Y, int s, cudaStream_t st) {
@@ -178,12 +157,12 @@ void scatter_owned(const int* own, int64_t n, const double2* Xsub, const double2
   scatter_t(own, n, Xsub, Q, Z, s, st);
 }
 void scatter_owned(const int* own, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
-                   cudaStream_t st) {
-  scatter_t(own, n, Xsub, Q, Z, s, st);
+                   cudaStream_t st, float4* Zdf, float2* Zf) {
+  scatter_t(own, n, Xsub, Q, Z, s, st, Zdf, Zf);
 }
 void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
-                   cudaStream_t st) {
-  scatter_t(own, n, Xsub, Q, Z, s, st);
+                   cudaStream_t st, float4* Zdf) {
+  scatter_t(own, n, Xsub, Q, Z, s, st, Zdf);
 }
 void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st) {
   scatter_t(own, n, Xsub, Q, Z, s, st);
@@ -235,25 +214,64 @@ void scatter_point_sources(double2* B, int64_t n, int s, const int* idx, const d
   if (nent) { k_point_sources<<<grid_for(nent, 128), 128, 0, st>>>(B, idx, val, nent); count_launch(); }
 }
 
-__global__ void k_to_rows(const double2* __restrict__ F, double2* __restrict__ B, int64_t n, int s) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g >= n * s) return;
-  int64_t r = g / s;
-  int c = (int)(g - r * s);
-  B[g] = F[(int64_t)c * n + r];
+// [s][n] <-> [n][s], through a tile of TR rows and up to TCOL columns
+// (blockIdx.y) so that both sides are read and written in full lines; to_rows
+// also in double-float (the operand of the product, without the FP64 rows in
+// between)
+constexpr int TR = 32, TCOL = 64;
+__device__ __forceinline__ void put_row(double2* p, double2 v) { *p = v; }
+__device__ __forceinline__ void put_row(float4* p, double2 v) { put_copy(p, v); }
+template <typename Out>
+__global__ void __launch_bounds__(256) k_to_rows(const double2* __restrict__ F, Out* __restrict__ B, int64_t n, int s) {
+  extern __shared__ double2 tile[];  // [columns][TR + 1]
+  const int64_t r0 = blockIdx.x * (int64_t)TR;
+  const int nr = (int)min((int64_t)TR, n - r0), c0 = blockIdx.y * TCOL, nc = min(TCOL, s - c0);
+  for (int e = threadIdx.x; e < TR * nc; e += blockDim.x) {
+    const int c = e / TR, r = e % TR;
+    if (r < nr) tile[c * (TR + 1) + r] = F[(int64_t)(c0 + c) * n + r0 + r];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nr * nc; e += blockDim.x) {
+    const int r = e / nc, c = e - r * nc;
+    put_row(B + (r0 + r) * s + c0 + c, tile[c * (TR + 1) + r]);
+  }
 }
-__global__ void k_from_rows(const double2* __restrict__ B, double2* __restrict__ F, int64_t n, int s) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g >= n * s) return;
-  int c = (int)(g / n);
-  int64_t r = g - (int64_t)c * n;
-  F[g] = B[r * s + c];
+__global__ void __launch_bounds__(256) k_from_rows(const double2* __restrict__ B, double2* __restrict__ F, int64_t n,
+                                                   int s) {
+  extern __shared__ double2 tile[];
+  const int64_t r0 = blockIdx.x * (int64_t)TR;
+  const int nr = (int)min((int64_t)TR, n - r0), c0 = blockIdx.y * TCOL, nc = min(TCOL, s - c0);
+  for (int e = threadIdx.x; e < nr * nc; e += blockDim.x) {
+    const int r = e / nc, c = e - r * nc;
+    tile[c * (TR + 1) + r] = B[(r0 + r) * s + c0 + c];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < TR * nc; e += blockDim.x) {
+    const int c = e / TR, r = e % TR;
+    if (r < nr) F[(int64_t)(c0 + c) * n + r0 + r] = tile[c * (TR + 1) + r];
+  }
 }
+// one column: the two layouts are the same
+__global__ void k_copy(const double2* __restrict__ X, double2* __restrict__ Y, int64_t count) {
+  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (g < count) Y[g] = X[g];
+}
+static dim3 tile_grid(int64_t n, int s) { return dim3(grid_for(n, TR), (s + TCOL - 1) / TCOL); }
+static size_t tile_bytes(int s) { return (size_t)std::min(s, TCOL) * (TR + 1) * sizeof(double2); }  // at most 33 KB
 void transpose_to_rows(const double2* F, double2* B, int64_t n, int s, cudaStream_t st) {
-  if (n * s) { k_to_rows<<<grid_for(n * s, 256), 256, 0, st>>>(F, B, n, s); count_launch(); }
+  if (n * s == 0) return;
+  if (s == 1) return cast_copy(F, B, n, st);
+  { k_to_rows<<<tile_grid(n, s), 256, tile_bytes(s), st>>>(F, B, n, s); count_launch(); }
+}
+void transpose_to_rows(const double2* F, float4* B, int64_t n, int s, cudaStream_t st) {
+  if (n * s == 0) return;
+  if (s == 1) return to_df(F, B, n, st);
+  { k_to_rows<<<tile_grid(n, s), 256, tile_bytes(s), st>>>(F, B, n, s); count_launch(); }
 }
 void transpose_from_rows(const double2* B, double2* F, int64_t n, int s, cudaStream_t st) {
-  if (n * s) { k_from_rows<<<grid_for(n * s, 256), 256, 0, st>>>(B, F, n, s); count_launch(); }
+  if (n * s == 0) return;
+  if (s == 1) return cast_copy(B, F, n, st);
+  { k_from_rows<<<tile_grid(n, s), 256, tile_bytes(s), st>>>(B, F, n, s); count_launch(); }
 }
 
 // debug_bounds: every entry a[i * stride] must lie in [lo, hi); the smallest
@@ -270,10 +288,6 @@ void check_index_range(const int* a, int64_t count, int stride, int64_t lo, int6
   if (count > 0 && a) { k_check_range<<<grid_for(count, 256), 256, 0, st>>>(a, count, stride, lo, hi, err, id); count_launch(); }
 }
 
-__global__ void k_copy(const double2* __restrict__ X, double2* __restrict__ Y, int64_t count) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g < count) Y[g] = X[g];
-}
 void cast_copy(const double2* X, double2* Y, int64_t count, cudaStream_t st) {
   if (count) { k_copy<<<grid_for(count, 256), 256, 0, st>>>(X, Y, count); count_launch(); }
 }

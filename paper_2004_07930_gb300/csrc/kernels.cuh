@@ -214,9 +214,10 @@ inline int64_t tc_tile_bytes(int nr, int nk) {  // nr output rows, nk reduction 
 }
 
 // --- sparse products ---
-// Y = A X (mode 0) or Y = B - A X (mode 1); X, Y, B row-major [n][s] complex
-void spmm_split(const DevSplitCsr& A, const double2* X, double2* Y, const double2* B, int s, int mode,
-                cudaStream_t st);
+// Y = A X, or Y = B - A X when B is given; X, Y, B row-major [n][s] complex; ordered: see spmm.cuh
+void spmm_split(const DevSplitCsr& A, const double2* X, double2* Y, const double2* B, int s, cudaStream_t st,
+                bool ordered = false);
+void spmm_split_cols(const DevSplitCsr& A, const double2* X, double2* Y, int s, cudaStream_t st);  // Y = A X, [s][n]
 // Y = R X for a real CSR R (rows x cols) on complex blocks
 void spmm_real(int64_t nrows, const int64_t* rp, const int32_t* col, const double* val, const double2* X,
                double2* Y, int s, cudaStream_t st);
@@ -228,13 +229,14 @@ int sweep_cols(int s);  // sweep.cu
 void gather_rows(const int* idx, int64_t nrows, const double2* X, double2* Y, int s, cudaStream_t st);
 void gather_rows(const int* idx, int64_t nrows, const double2* X, float2* Y, int s, cudaStream_t st);
 void gather_rows(const int* idx, int64_t nrows, const float2* X, float2* Y, int s, cudaStream_t st);
-// Z[r][:] = Xsub[own[r]][:] (+ Q[r][:]), in Z's precision (Q may be NULL)
+// Z[r][:] = Xsub[own[r]][:] (+ Q[r][:]), in Z's precision (Q may be NULL); Zdf: Z in double-float beside it,
+// Zf: the FP32 sub-vector values themselves (Z without Q)
 void scatter_owned(const int* own, int64_t n, const double2* Xsub, const double2* Q, double2* Z, int s,
                    cudaStream_t st);
 void scatter_owned(const int* own, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
-                   cudaStream_t st);
+                   cudaStream_t st, float4* Zdf = nullptr, float2* Zf = nullptr);
 void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
-                   cudaStream_t st);
+                   cudaStream_t st, float4* Zdf = nullptr);
 void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st);
 
 // --- multifrontal ---
@@ -280,10 +282,14 @@ struct DevKrylov {
 // --- double-float products (mixed form, emulated FP64; df.cu) ---
 // X [count] complex FP64 -> (re_hi, re_lo, im_hi, im_lo)
 void to_df(const double2* X, float4* Y, int64_t count, cudaStream_t st);
-// Y = A X (mode 0) or Y = B - A X (mode 1) with X in double-float, A's double-float values;
-// with Ydf, A X in double-float instead of Y
-void spmm_split_df(const DevSplitCsr& A, const float4* X, double2* Y, const double2* B, int s, int mode,
-                   cudaStream_t st, float4* Ydf = nullptr);
+// Products with A's double-float values; X in double-float, or in FP32 (z of the one-level
+// preconditioner and of the coarse ORAS has no more)
+void spmm_split_df(const DevSplitCsr& A, const float4* X, double2* Y, const double2* B, int s,
+                   cudaStream_t st);                                                                // A X or B - A X
+void spmm_split_df_cols(const DevSplitCsr& A, const float4* X, double2* Y, int s, cudaStream_t st);  // A X, [s][n]
+void spmm_split_df(const DevSplitCsr& A, const float4* X, float4* Y, int s, cudaStream_t st);        // A X in double-float
+void spmm_split_df(const DevSplitCsr& A, const float2* X, double2* Y, int s, cudaStream_t st);
+void spmm_split_df(const DevSplitCsr& A, const float2* X, float4* Y, int s, cudaStream_t st, bool ordered = false);
 
 // Y = R X for a real CSR R with double-float values, X in double-float, Y in FP64
 void spmm_real_df(int64_t nrows, const int64_t* rp, const int32_t* col, const float2* val, const float4* X,
@@ -350,6 +356,7 @@ void cast_f2d(const float2* X, double2* Y, int64_t count, cudaStream_t st);
 void scatter_point_sources(double2* B, int64_t n, int s, const int* idx, const double2* val, int nent,
                            cudaStream_t st);
 void transpose_to_rows(const double2* F, double2* B, int64_t n, int s, cudaStream_t st);    // [s][n] -> [n][s]
+void transpose_to_rows(const double2* F, float4* B, int64_t n, int s, cudaStream_t st);     // in double-float
 void transpose_from_rows(const double2* B, double2* F, int64_t n, int s, cudaStream_t st);  // [n][s] -> [s][n]
 void cast_copy(const double2* X, double2* Y, int64_t count, cudaStream_t st);
 // debug_bounds: atomicMin(err, id) if some a[i * stride], i < count, lies outside [lo, hi)

@@ -22,6 +22,7 @@
 
 #include "df.cuh"
 #include "kernels.cuh"
+#include "spmm.cuh"
 
 namespace hz {
 
@@ -571,65 +572,28 @@ void krylov_update(DevKrylov& K, void* X, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // FP32 coarse-level helpers (mixed form): SpMM with float values, precision casts
 // ---------------------------------------------------------------------------
-// Y = A X, or Y = B - A X when B is given (FP32 values and blocks)
-__global__ void k_spmm_split_f32(int64_t n, int s, const int64_t* __restrict__ rp_re, const int32_t* __restrict__ col_re,
-                                 const float* __restrict__ val_re, const int64_t* __restrict__ rp_im,
-                                 const int32_t* __restrict__ col_im, const float* __restrict__ val_im,
-                                 const float2* __restrict__ X, float2* __restrict__ Y, const float2* __restrict__ B) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  int c = (int)(g - r * s);
-  if (r >= n) return;
-  float ar = 0.f, ai = 0.f;
-  #pragma unroll 4
-  for (int64_t p = rp_re[r], pe = rp_re[r + 1]; p < pe; ++p) {
-    float a = val_re[p];
-    float2 x = X[(int64_t)col_re[p] * s + c];
-    ar = fmaf(a, x.x, ar);
-    ai = fmaf(a, x.y, ai);
+namespace {
+struct OutRowsF {  // Y = A X, or B - A X
+  float2* Y;
+  const float2* B;
+  int s;
+  __device__ __forceinline__ void operator()(int64_t r, int c, float2 y) const {
+    const int64_t g = r * s + c;
+    if (B) {
+      const float2 b = B[g];
+      y = make_float2(b.x - y.x, b.y - y.y);
+    }
+    Y[g] = y;
   }
-  #pragma unroll 4
-  for (int64_t p = rp_im[r], pe = rp_im[r + 1]; p < pe; ++p) {
-    float b = val_im[p];
-    float2 x = X[(int64_t)col_im[p] * s + c];
-    ar = fmaf(-b, x.y, ar);
-    ai = fmaf(b, x.x, ai);
-  }
-  if (B) {
-    const float2 b = B[g];
-    Y[g] = make_float2(b.x - ar, b.y - ai);
-  } else {
-    Y[g] = make_float2(ar, ai);
-  }
-}
+};
+}  // namespace
 
 void spmm_split_f32(const DevSplitCsr& A, const float2* X, float2* Y, int s, cudaStream_t st, const float2* B) {
-  int64_t work = A.n * s;
-  if (work == 0) return;
-  { k_spmm_split_f32<<<grid_for(work, 256), 256, 0, st>>>(A.n, s, A.rp_re, A.col_re, A.val_re_f, A.rp_im, A.col_im,
-                                                        A.val_im_f, X, Y, B); count_launch(); }
+  spmm_launch<SpF32>(A.n, s, A.rp_re, A.col_re, A.val_re_f, A.rp_im, A.col_im, A.val_im_f, X, OutRowsF{Y, B, s}, st, true);
 }
-
-__global__ void k_spmm_real_f32(int64_t n, int s, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                const float* __restrict__ val, const float2* __restrict__ X, float2* __restrict__ Y) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t r = g / s;
-  int c = (int)(g - r * s);
-  if (r >= n) return;
-  float ar = 0.f, ai = 0.f;
-  #pragma unroll 4
-  for (int64_t p = rp[r], pe = rp[r + 1]; p < pe; ++p) {
-    float a = val[p];
-    float2 x = X[(int64_t)col[p] * s + c];
-    ar = fmaf(a, x.x, ar);
-    ai = fmaf(a, x.y, ai);
-  }
-  Y[g] = make_float2(ar, ai);
-}
-
 void spmm_real_f32(int64_t nrows, const int64_t* rp, const int32_t* col, const float* val, const float2* X,
                    float2* Y, int s, cudaStream_t st) {
-  if (nrows * s) { k_spmm_real_f32<<<grid_for(nrows * s, 256), 256, 0, st>>>(nrows, s, rp, col, val, X, Y); count_launch(); }
+  spmm_launch<SpF32>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRowsF{Y, nullptr, s}, st, true);
 }
 
 __global__ void k_d2f(const double2* __restrict__ X, float2* __restrict__ Y, int64_t count) {

@@ -79,7 +79,7 @@ extern "C" int hz_apply_A_noalloc(hz_ctx* ctx, const double* X, double* Y, int32
   double2* B = scratch;                // [n][s] input rows
   double2* R = scratch + kMaxEntries;  // [n][s] product rows
   transpose_to_rows(reinterpret_cast<const double2*>(X), B, n, s, st);
-  spmm_split(*A, B, R, nullptr, s, 0, st);
+  spmm_split(*A, B, R, nullptr, s, st);
   transpose_from_rows(R, reinterpret_cast<double2*>(Y), n, s, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
