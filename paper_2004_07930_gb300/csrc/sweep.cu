@@ -31,7 +31,11 @@
 //
 // What bounds it: on the 5 Hz workload (0.95M dofs, 64 subdomains, 16
 // columns) the FP32 FMA pipe: 444M factor entries, 114 GFLOP per
-// application, 1.5 ms at the pipe's 74.8 TFLOP/s; with one column HBM: 7.1 GB, 1.05 ms.
+// application, 1.5 ms at the pipe's 74.8 TFLOP/s; with one column HBM: 7.1 GB,
+// 1.05 ms. Measured, whole preconditioner: 4.05 ms (tiles of 64 x 64 per CTA,
+// one output row per thread: 7.16) and 1.69 ms (2.00). The leaf level runs at
+// 52-55 % of the pipe; the middle levels, 1-10 K small fronts each, spend
+// 30-55 us on the latency of task, indices, inputs and factors in turn.
 //
 // FP64 has one pipe per scheduler that takes a warp's multiply-add every 64
 // clocks (1.2 TFLOP/s over the 608 schedulers), so that a short level must
@@ -72,19 +76,21 @@ struct SwV {
 // Lanes of a warp: CL lanes share a row, each with CPT columns; RG row sets of
 // up to RPT rows each. FP32 works on row pairs (packed multiply-adds). FP64
 // with one column gives the real and the imaginary part to two lanes.
-// Staging: RPP input rows per pass of the CTA, U passes (CH rows) at a time
-// when the input does not fit.
-template <typename V, int S>
+// Staging: a thread moves SPT columns (FP32: 16 bytes) of a row, RPP rows per
+// pass of the CTA, U passes (CH rows) at a time where the input streams by.
+template <typename V, int S, bool FWD>
 struct SwS {
   static constexpr bool F32 = sizeof(V) == 8;
   static constexpr bool SPLIT = !F32 && S == 1;
   static constexpr int RPT = F32 ? (S == 16 ? 4 : 2) : (S == 16 ? 4 : (S == 8 ? 2 : 1));
   static constexpr int CPT = F32 ? (S >= 8 ? 2 : 1) : (S >= 4 ? 2 : 1);
-  static constexpr int CLS = S / CPT;  // lanes per staged row
-  static constexpr int CL = SPLIT ? 2 : CLS;
+  static constexpr int CL = SPLIT ? 2 : S / CPT;
   static constexpr int RG = MF_GR / RPT;  // FP64: row sets of a warp
+  static constexpr int SPT = F32 ? (S >= 2 ? 2 : 1) : CPT;
+  static constexpr int CLS = S / SPT;
   static constexpr int RPP = SW_THREADS / CLS;
-  static constexpr int U = RPP < 32 ? 32 / RPP : 1;
+  static constexpr int WANT = F32 && !FWD ? 64 : 32;  // the forward rows pass through registers
+  static constexpr int U = RPP < WANT ? WANT / RPP : 1;
   static constexpr int CH = U * RPP;
 };
 
@@ -150,6 +156,7 @@ struct SweepArgs {
   V* Xsub;
   V* Wout;
   int s;               // row length of Xsub and Wout (sweep_cols)
+  int kids;            // some front of the level has children
 };
 
 // Packed pairs of FP32 numbers: fma.rn.f32x2 rounds each half like a scalar
@@ -180,7 +187,7 @@ template <typename V, int S>
 struct SwAcc;
 template <int S>
 struct SwAcc<float2, S> {
-  using L = SwS<float2, S>;
+  using L = SwS<float2, S, true>;
   static constexpr int P = L::RPT / 2, CPT = L::CPT;
   pair2 re[P][CPT], im[P][CPT];
   __device__ __forceinline__ void zero() {
@@ -259,7 +266,7 @@ struct SwAcc<float2, S> {
 };
 template <int S>
 struct SwAcc<double2, S> {
-  using L = SwS<double2, S>;
+  using L = SwS<double2, S, true>;
   static constexpr int RPT = L::RPT, CPT = L::CPT, RG = L::RG;
   double2 v[RPT][CPT];
   __device__ __forceinline__ void zero() {
@@ -334,8 +341,8 @@ struct SwAcc<double2, S> {
 template <typename V, int S, bool FWD, bool STREAM, bool KS, typename Wait>
 __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepTask& T, int c0, unsigned char* smem,
                                            Wait&& wait) {
-  using L = SwS<V, S>;
-  constexpr int CPT = L::CPT, CL = L::CL, CLS = L::CLS, RPT = L::RPT;
+  using L = SwS<V, S, FWD>;
+  constexpr int CPT = L::CPT, SPT = L::SPT, CL = L::CL, CLS = L::CLS, RPT = L::RPT;
   constexpr int KC = KS ? 2048 / (MF_GR * (int)sizeof(V)) : SwV<V, FWD, STREAM>::KC;  // KS: the same in every form
   constexpr int STAGE = SwV<V, FWD, STREAM>::STAGE, BYTES = SwV<V, FWD, STREAM>::BYTES;
   constexpr int U = L::U, RPP = L::RPP, CH = L::CH;
@@ -349,8 +356,19 @@ __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepT
   const int lo = FWD ? 0 : MF_GR * T.g0;
   const int hi = FWD ? min(k, MF_GR * gend) : f;
   const int rg = lane / CL, col = L::SPLIT ? 0 : (lane % CL) * CPT;  // lane's row set and first column
-  const int c = c0 + col;
-  const int tr = tid / CLS, scol = (tid % CLS) * CPT;  // staging: input row of a pass, first column
+  const int tr = tid / CLS, scol = (tid % CLS) * SPT;  // staging: input row of a pass, first column
+  const uint32_t pitch = (uint32_t)s * sizeof(V);      // bytes of a row
+  // row r of Xsub or Wout, from column q of the task's on
+  auto xrow = [&](int r, int q) {
+    return reinterpret_cast<V*>(reinterpret_cast<char*>(A.Xsub + c0 + q) + (uint64_t)(uint32_t)r * pitch);
+  };
+  auto wrow = [&](int r, int q) {
+    return reinterpret_cast<V*>(reinterpret_cast<char*>(A.Wout + c0 + q) + (uint64_t)(uint32_t)r * pitch);
+  };
+  V* const own = A.Wout + T.row * s + c0;               // the front's own rows
+  auto orow = [&](int r, int q) {
+    return reinterpret_cast<V*>(reinterpret_cast<char*>(own + q) + (uint32_t)r * pitch);
+  };
 
   // ring: stages of the warp's groups g0 + warp, + SW_NW, ... in order
   int ig = KS ? T.g0 : T.g0 + warp, il = 0, inb = 0, islot = 0;  // group, bytes of it left, bytes per full stage, slot
@@ -390,45 +408,56 @@ __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepT
 #pragma unroll
   for (int i = 0; i < SW_NST - 1; ++i) issue();
 
-  // input rows lb + u RPP + tr, u < N: their sources, then their values
+  // input rows lb + u RPP + tr, u < N: their sources, then their values. The
+  // backward rows are plain copies (FP32: cp.async, 16 columns of the 5 Hz
+  // workload 4.28 -> 4.05 ms with the wider staging; FP64 gained nothing, as a
+  // wait for them also waits for the ring); the forward ones are sums of up to
+  // three rows and pass through registers, like one column's 8-byte rows.
+  constexpr bool COPY = !FWD && L::F32 && SPT * sizeof(V) == 16;
   auto load_idx = [&](int lb, auto& xr, auto& cc) {
     constexpr int N = sizeof(xr) / sizeof(int);
 #pragma unroll
     for (int u = 0; u < N; ++u) {
       const int l = lb + u * RPP + tr;
       xr[u] = -1;
-      cc[u] = make_int2(-1, -1);
+      if (FWD) cc[u] = make_int2(-1, -1);
       if (l < hi) {
         if (FWD || l >= k) xr[u] = __ldg(A.rows + T.row + l);
-        if (FWD) cc[u] = __ldg(A.csrc + T.row + l);
+        if (FWD && A.kids) cc[u] = __ldg(A.csrc + T.row + l);
       }
     }
   };
-  auto load_val = [&](int lb, const auto& xr, const auto& cc, auto& v, auto& w0, auto& w1) {
+  auto load_val = [&](int lb, const auto& xr, const auto& cc, auto& v, auto& w0, auto& w1, V* dst) {
     constexpr int N = sizeof(xr) / sizeof(int);
 #pragma unroll
     for (int u = 0; u < N; ++u) {
       const int l = lb + u * RPP + tr;
       if (l < hi) {
-        ld_cols<CPT>(xr[u] >= 0 ? A.Xsub + (int64_t)xr[u] * s + c0 + scol : A.Wout + (T.row + l) * s + c0 + scol, v[u]);
-        if (FWD) {
+        const V* src = FWD || xr[u] >= 0 ? xrow(xr[u], scol) : orow(l, scol);
+        if (COPY) {
+          cp_async16((uint32_t)__cvta_generic_to_shared(dst + (u * RPP + tr) * S + scol), src);
+        } else {
+          ld_cols<SPT>(src, v[u]);
+          if (FWD && A.kids) {
 #pragma unroll
-          for (int p = 0; p < CPT; ++p) w0[u][p] = w1[u][p] = c_zero<V>();
-          if (cc[u].x >= 0) ld_cols<CPT>(A.Wout + (int64_t)cc[u].x * s + c0 + scol, w0[u]);
-          if (cc[u].y >= 0) ld_cols<CPT>(A.Wout + (int64_t)cc[u].y * s + c0 + scol, w1[u]);
+            for (int p = 0; p < SPT; ++p) w0[u][p] = w1[u][p] = c_zero<V>();
+            if (cc[u].x >= 0) ld_cols<SPT>(wrow(cc[u].x, scol), w0[u]);
+            if (cc[u].y >= 0) ld_cols<SPT>(wrow(cc[u].y, scol), w1[u]);
+          }
         }
       }
     }
   };
   auto store_val = [&](V* dst, int lb, auto& v, const auto& w0, const auto& w1) {  // row lb at dst[0]
-    constexpr int N = sizeof(v) / (CPT * sizeof(V));
+    constexpr int N = sizeof(v) / (SPT * sizeof(V));
+    if (COPY) return;
 #pragma unroll
     for (int u = 0; u < N; ++u) {
       const int l = u * RPP + tr;
       if (lb + l < hi) {
 #pragma unroll
-        for (int p = 0; p < CPT; ++p) {
-          if (FWD) v[u][p] = c_add(c_add(v[u][p], w0[u][p]), w1[u][p]);
+        for (int p = 0; p < SPT; ++p) {
+          if (FWD && A.kids) v[u][p] = c_add(c_add(v[u][p], w0[u][p]), w1[u][p]);
           dst[l * S + scol + p] = v[u][p];
         }
       }
@@ -444,37 +473,44 @@ __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepT
     load_idx(lo, xr, cc);
     if (!wait()) return false;
     for (int lb = lo; lb < end; lb += NF * RPP) {
-      V v[NF][CPT], w0[NF][CPT], w1[NF][CPT];
-      load_val(lb, xr, cc, v, w0, w1);
+      V v[NF][SPT], w0[NF][SPT], w1[NF][SPT];
+      load_val(lb, xr, cc, v, w0, w1, bs + (lb - lo) * S);
       if (lb + NF * RPP < end) load_idx(lb + NF * RPP, xr, cc);
       store_val(bs + (lb - lo) * S, lb, v, w0, w1);
     }
   }
+  if (COPY) {
+    cp_async_commit();
+    cp_async_wait<0>();
+  }
   int xr[U];
   int2 cc[U];
-  V v[U][CPT], w0[U][CPT], w1[U][CPT];
+  V v[U][SPT], w0[U][SPT], w1[U][SPT];
   if (STREAM) load_idx(end, xr, cc);
 
   SwAcc<V, S> acc, tot;
   acc.zero();
-  tot.zero();
+  if (!L::F32) tot.zero();
   int cg = KS ? T.g0 : T.g0 + warp, slot = 0, used = 0;  // group, ring slot being read, indices of it already used
   int ck = (FWD ? 0 : MF_GR * cg) + (KS ? warp * KC : 0);  // next reduction index of the group
   bool part = false;                         // `tot` holds the earlier chunks of the group
-  // where the rows of the group go (backward), or the children's updates that join them (forward)
-  int xo[RPT];
-  int2 ce[RPT];
+  // the lane's rows of the group: the first one, how many; where they go (backward), or the children's
+  // updates that join them (forward)
+  int r0 = 0, nv = 0, xo[FWD ? 1 : RPT];
+  int2 ce[FWD ? RPT : 1];
   auto targets = [&]() {
-    const int rpt = SwAcc<V, S>::rows(mf_group_rows(nout, min(cg, gend - 1)));
+    const int nrp = mf_group_rows(nout, min(cg, gend - 1)), rpt = SwAcc<V, S>::rows(nrp);
+    r0 = MF_GR * cg + rg * rpt;
+    nv = rg * rpt < nrp ? max(0, min(rpt, nout - r0)) : 0;
+    if (cg >= gend) nv = 0;
 #pragma unroll
     for (int i = 0; i < RPT; ++i) {
-      const int r = MF_GR * cg + rg * rpt + i;
-      const bool in = cg < gend && i < rpt && r < nout && rg * rpt < MF_GR;
-      xo[i] = -1;
-      ce[i] = make_int2(-1, -1);
-      if (!FWD && in) xo[i] = __ldg(A.rows + T.row + r);
-      if (FWD && in) xo[i] = r;
-      if (FWD && in && r >= k) ce[i] = __ldg(A.csrc + T.row + r);
+      if (FWD) {
+        ce[i] = make_int2(-1, -1);
+        if (A.kids && i < nv && r0 + i >= k) ce[i] = __ldg(A.csrc + T.row + r0 + i);
+      } else {
+        if (i < nv) xo[i] = __ldg(A.rows + T.row + r0 + i);
+      }
     }
   };
   targets();
@@ -483,7 +519,7 @@ __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepT
     __syncthreads();
     const bool more = STREAM && end < hi;
     if (more) {
-      load_val(end, xr, cc, v, w0, w1);
+      load_val(end, xr, cc, v, w0, w1, buf == bs ? bs + CH * S : bs);  // joins the next ring stage's copies
       load_idx(end + CH, xr, cc);
     }
     while (cg < gend) {
@@ -493,7 +529,10 @@ __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepT
       const V* b = buf + col;
       while (ck < kstop) {
         if (!KS && (ck & (MF_CHUNK - 1)) == 0 && ck > kfirst) {  // a chunk is complete
-          tot.add(acc);
+          if (part || !L::F32)
+            tot.add(acc);
+          else
+            tot = acc;
           acc.zero();
           part = true;
         }
@@ -527,51 +566,56 @@ __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepT
       if (part) {
         tot.add(acc);
         acc = tot;
-        tot.zero();
+        if (!L::F32) tot.zero();
       }
+      const int nst = L::SPLIT && (lane & 1) ? 0 : nv;  // rows the lane writes
       if (!FWD) {
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
           V o[CPT];
 #pragma unroll
           for (int q = 0; q < CPT; ++q) o[q] = acc.get(i, q);
-          if (xo[i] >= 0 && !(L::SPLIT && (lane & 1))) st_cols<CPT>(A.Xsub + (int64_t)xo[i] * s + c, o);
+          if (i < nst) st_cols<CPT>(xrow(xo[i], col), o);
         }
       } else {
-        V o[RPT][CPT];
+        // rows at a time: all their loads, then their sums. FP64 adds zeros where there is no child: a
+        // branch around each addition left its loads one behind the other (cube, 3 columns: 0.71 -> 0.64 ms)
+        constexpr int NB = L::F32 ? (RPT < 2 ? 1 : 2) : RPT;
 #pragma unroll
-        for (int i = 0; i < RPT; ++i)
+        for (int i0 = 0; i0 < RPT; i0 += NB) {
+          V o[NB][CPT], x0[NB][CPT], x1[NB][CPT];
 #pragma unroll
-          for (int q = 0; q < CPT; ++q) o[i][q] = acc.get(i, q);
-        if (MF_GR * cg < k) {  // a group with pivot rows
+          for (int h = 0; h < NB; ++h) {
+            if (!L::F32) {
 #pragma unroll
-          for (int i = 0; i < RPT; ++i)
-            if (xo[i] >= 0 && xo[i] < k) {
-              const V di = __ldg(A.Dinv + T.d + xo[i]);
-#pragma unroll
-              for (int q = 0; q < CPT; ++q) o[i][q] = part ? mul_dinv<true>(o[i][q], di) : mul_dinv<false>(o[i][q], di);
+              for (int q = 0; q < CPT; ++q) x0[h][q] = x1[h][q] = c_zero<V>();
             }
-        }
-        bool kids = false;
+            if (ce[i0 + h].x >= 0) ld_cols<CPT>(wrow(ce[i0 + h].x, col), x0[h]);
+            if (ce[i0 + h].y >= 0) ld_cols<CPT>(wrow(ce[i0 + h].y, col), x1[h]);
 #pragma unroll
-        for (int i = 0; i < RPT; ++i) kids |= ce[i].x >= 0;
-        if (__any_sync(0xffffffffu, kids)) {
-          V x0[RPT][CPT], x1[RPT][CPT];
+            for (int q = 0; q < CPT; ++q) o[h][q] = acc.get(i0 + h, q);
+          }
+          if (MF_GR * cg < k) {  // a group with pivot rows
 #pragma unroll
-          for (int i = 0; i < RPT; ++i) {
+            for (int h = 0; h < NB; ++h)
+              if (i0 + h < nv && r0 + i0 + h < k) {
+                const V di = __ldg(A.Dinv + T.d + r0 + i0 + h);
 #pragma unroll
-            for (int q = 0; q < CPT; ++q) x0[i][q] = x1[i][q] = c_zero<V>();
-            if (ce[i].x >= 0) ld_cols<CPT>(A.Wout + (int64_t)ce[i].x * s + c, x0[i]);
-            if (ce[i].y >= 0) ld_cols<CPT>(A.Wout + (int64_t)ce[i].y * s + c, x1[i]);
+                for (int q = 0; q < CPT; ++q)
+                  o[h][q] = part ? mul_dinv<true>(o[h][q], di) : mul_dinv<false>(o[h][q], di);
+              }
           }
 #pragma unroll
-          for (int i = 0; i < RPT; ++i)
+          for (int h = 0; h < NB; ++h) {
+            if (!L::F32 || ce[i0 + h].x >= 0)
 #pragma unroll
-            for (int q = 0; q < CPT; ++q) o[i][q] = c_add(c_add(o[i][q], x0[i][q]), x1[i][q]);
+              for (int q = 0; q < CPT; ++q) o[h][q] = c_add(o[h][q], x0[h][q]);
+            if (!L::F32 || ce[i0 + h].y >= 0)
+#pragma unroll
+              for (int q = 0; q < CPT; ++q) o[h][q] = c_add(o[h][q], x1[h][q]);
+            if (i0 + h < nst) st_cols<CPT>(orow(r0 + i0 + h, col), o[h]);
+          }
         }
-#pragma unroll
-        for (int i = 0; i < RPT; ++i)
-          if (xo[i] >= 0 && !(L::SPLIT && (lane & 1))) st_cols<CPT>(A.Wout + (T.row + xo[i]) * s + c, o[i]);
       }
       acc.zero();
       part = false;
@@ -582,6 +626,10 @@ __device__ __forceinline__ bool sweep_task_t(const SweepArgs<V>& A, const SweepT
     if (!more) break;
     buf = buf == bs ? bs + CH * S : bs;
     store_val(buf, end, v, w0, w1);
+    if (COPY) {
+      cp_async_commit();
+      cp_async_wait<0>();
+    }
     base = end;
     end = min(end + CH, hi);
   }
@@ -596,14 +644,14 @@ __device__ __forceinline__ bool sweep_task(const SweepArgs<V>& A, const SweepTas
 }
 
 // CTAs per SM to leave registers for
-template <typename V, int S, bool STREAM>
+template <typename V, int S, bool FWD, bool STREAM>
 constexpr int sw_min_blocks() {
-  return sizeof(V) == 16 ? 2 : (STREAM ? 4 : (S <= 2 ? 8 : 6));
+  return sizeof(V) == 16 ? 2 : (STREAM ? 4 : (S <= 2 ? 8 : (FWD && S == 16 ? 5 : 6)));
 }
 
 // One level of one sweep: blockIdx = task * (column blocks) + column block.
 template <typename V, int S, bool FWD, bool STREAM>
-__global__ void __launch_bounds__(SW_THREADS, sw_min_blocks<V, S, STREAM>()) k_sweep_level(SweepArgs<V> A, int ncb) {
+__global__ void __launch_bounds__(SW_THREADS, sw_min_blocks<V, S, FWD, STREAM>()) k_sweep_level(SweepArgs<V> A, int ncb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
   const int ti = blockIdx.x / ncb;
@@ -649,7 +697,7 @@ __device__ __forceinline__ bool sw_wait(const int* p, int target) {
 }
 
 template <typename V, int S, bool FWD>
-__global__ void __launch_bounds__(SW_THREADS, sw_min_blocks<V, S, true>()) k_sweep_all(
+__global__ void __launch_bounds__(SW_THREADS, sw_min_blocks<V, S, FWD, true>()) k_sweep_all(
     SweepArgs<V> A, int ncb, int ntasks, const int* __restrict__ front_tasks, const int* __restrict__ dep,
     const int* __restrict__ nchild, int* __restrict__ cnt, int nfronts, int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -696,8 +744,8 @@ size_t sw_smem(int rows) {
   return (size_t)SW_NW * SW_NST * SwV<V, FWD, STREAM>::BYTES + (size_t)rows * S * sizeof(V);
 }
 
-// The tasks of level l. A level whose longest reduction fits MF_RES rows
-// stages its inputs whole.
+// The tasks of level l. A level whose longest reduction fits stages its
+// inputs whole.
 template <typename V, int S, bool FWD>
 void launch_level(const DevMF& mf, SweepArgs<V>& A, int l, cudaStream_t st) {
   const int* ptr = FWD ? mf.ftask_ptr_h : mf.btask_ptr_h;
@@ -707,7 +755,7 @@ void launch_level(const DevMF& mf, SweepArgs<V>& A, int l, cudaStream_t st) {
   if (rows <= MF_RES)
     launch_k(true, k_sweep_level<V, S, FWD, false>, grid, SW_THREADS, sw_smem<V, S, FWD, false>(rows), st, A, ncb);
   else
-    launch_k(true, k_sweep_level<V, S, FWD, true>, grid, SW_THREADS, sw_smem<V, S, FWD, true>(2 * SwS<V, S>::CH), st, A,
+    launch_k(true, k_sweep_level<V, S, FWD, true>, grid, SW_THREADS, sw_smem<V, S, FWD, true>(2 * SwS<V, S, FWD>::CH), st, A,
              ncb);
 }
 
@@ -719,6 +767,7 @@ void sweep_level(const DevMF& mf, SweepArgs<V>& A, int l, cudaStream_t st) {
   const int* ptr = FWD ? mf.ftask_ptr_h : mf.btask_ptr_h;
   if (ptr[l + 1] == ptr[l]) return;
   A.M = (const V*)(FWD ? mf.M : mf.MT);
+  A.kids = l > 0;  // level 0 holds the leaves
   const int64_t groups = (FWD ? mf.fgroups_h : mf.bgroups_h)[l];
   int w = A.s % 16 == 0 ? 16 : (A.s % 8 == 0 ? 8 : A.s);
   while (w > 4 && groups * (A.s / w) < 1216) w /= 2;
@@ -736,11 +785,12 @@ void sweep_all(const DevMF& mf, SweepArgs<V>& A, cudaStream_t st) {
   const int ncb = A.s / S;
   const int nt = (FWD ? mf.ftask_ptr_h : mf.btask_ptr_h)[mf.nlevels];
   if (nt == 0) return;
-  const size_t shm = sw_smem<V, S, FWD, true>(2 * SwS<V, S>::CH);
+  const size_t shm = sw_smem<V, S, FWD, true>(2 * SwS<V, S, FWD>::CH);
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep_all<V, S, FWD>, SW_THREADS, shm);
+  A.kids = 1;
   A.tasks = FWD ? mf.ftasks : mf.btasks_top;
   A.M = (const V*)(FWD ? mf.M : mf.MT);
   cudaMemsetAsync(mf.cnt, 0, (size_t)(1 + 2 * mf.nfronts) * sizeof(int), st);
@@ -781,7 +831,7 @@ void solve_v(DevMF& mf, V* Xsub, int cols, cudaStream_t st) {
 
 template <typename V, int S, bool FWD>
 void attrs_sf() {
-  const int whole = (int)sw_smem<V, S, FWD, false>(MF_RES), stream = (int)sw_smem<V, S, FWD, true>(2 * SwS<V, S>::CH);
+  const int whole = (int)sw_smem<V, S, FWD, false>(MF_RES), stream = (int)sw_smem<V, S, FWD, true>(2 * SwS<V, S, FWD>::CH);
   cudaFuncSetAttribute(k_sweep_level<V, S, FWD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, whole);
   cudaFuncSetAttribute(k_sweep_level<V, S, FWD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, stream);
   cudaFuncSetAttribute(k_sweep_all<V, S, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, stream);
