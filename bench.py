@@ -726,7 +726,7 @@ def main():
         pers = r.get("persistent_sweeps", 0) == 1
         kern = ("fine local solves (tcgen05 sweep tiles, 3xTF32 split, FP32 accumulation in TMEM, one launch per "
                 "level)" if tc_on else "fine local solves (SIMT complex FP32 sweep tiles, %s)" %
-                ("k_mf_sweep: one launch per sweep over all levels" if pers else "k_mf_tile + k_mf_reduce per level"))
+                ("k_sweep_all: one launch per sweep over all levels" if pers else "k_sweep_level per level"))
         # a sweep reads each factor entry once per application: HBM is the roof of the
         # tensor-core form; the SIMT FP32 rate (16 flops per factor byte at s = 16) is given beside it
         roof = {"bound": "hbm", "achieved": hbm_achieved, "peak": hbm, "unit": "GB/s", "frac": hbm_achieved / hbm,

@@ -17,7 +17,8 @@
 // the mixed form's FP32 local solves.
 //
 // Layouts: a complex FP64 block [n][s] double2 becomes [n][s] float4
-// (re_hi, re_lo, im_hi, im_lo), 16 bytes per entry like the FP64 block; the
+// (re_hi, im_hi, re_lo, im_lo), 16 bytes per entry like the FP64 block, the
+// operand pairs of the packed arithmetic; the
 // real values of a split CSR matrix become float2 (hi, lo) per nonzero.
 #include <cuda_runtime.h>
 
@@ -36,17 +37,18 @@ __global__ void k_to_df(const double2* __restrict__ X, float4* __restrict__ Y, i
   if (g >= count) return;
   const double2 x = X[g];
   const float2 r = df_split(x.x), i = df_split(x.y);
-  Y[g] = make_float4(r.x, r.y, i.x, i.y);
+  Y[g] = make_float4(r.x, i.x, r.y, i.y);
 }
 
 namespace {
+template <typename P>
 struct OutRows {  // Y = A X, or B - A X
   double2* Y;
   const double2* B;
   int s;
-  __device__ __forceinline__ void operator()(int64_t r, int c, float4 a) const {
+  __device__ __forceinline__ void operator()(int64_t r, int c, typename P::Acc a) const {
     const int64_t g = r * s + c;
-    const double2 y = SpDf<float4>::to_d(a);
+    const double2 y = P::to_d(a);
     if (B) {
       const double2 b = B[g];
       Y[g] = make_double2(b.x - y.x, b.y - y.y);
@@ -55,20 +57,23 @@ struct OutRows {  // Y = A X, or B - A X
     }
   }
 };
+template <typename P>
 struct OutCols {  // Y = A X with the columns contiguous, [s][n]
   double2* Y;
   int64_t n;
-  __device__ __forceinline__ void operator()(int64_t r, int c, float4 a) const {
-    Y[(int64_t)c * n + r] = SpDf<float4>::to_d(a);
+  __device__ __forceinline__ void operator()(int64_t r, int c, typename P::Acc a) const {
+    Y[(int64_t)c * n + r] = P::to_d(a);
   }
 };
-struct OutDf {  // Y = A X in double-float, renormalised
+template <typename P>
+struct OutDf {  // Y = A X in double-float, renormalised, (re hi, re lo, im hi, im lo)
   float4* Y;
   int s;
-  __device__ __forceinline__ void operator()(int64_t r, int c, float4 a) const {
-    df_norm(a.x, a.y);
-    df_norm(a.z, a.w);
-    Y[r * s + c] = a;
+  __device__ __forceinline__ void operator()(int64_t r, int c, typename P::Acc a) const {
+    float4 y = P::parts(a);
+    df_norm(y.x, y.y);
+    df_norm(y.z, y.w);
+    Y[r * s + c] = y;
   }
 };
 template <typename XT, typename Out>
@@ -79,7 +84,8 @@ void spmm_df(const DevSplitCsr& A, const XT* X, Out out, int s, cudaStream_t st,
 
 void spmm_real_df(int64_t nrows, const int64_t* rp, const int32_t* col, const float2* val, const float4* X,
                   double2* Y, int s, cudaStream_t st) {
-  spmm_launch<SpDf<float4>>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRows{Y, nullptr, s}, st, true);
+  spmm_launch<SpDf<float4>>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X,
+                            OutRows<SpDf<float4>>{Y, nullptr, s}, st, true);
 }
 
 void to_df(const double2* X, float4* Y, int64_t count, cudaStream_t st) {
@@ -87,19 +93,19 @@ void to_df(const double2* X, float4* Y, int64_t count, cudaStream_t st) {
 }
 
 void spmm_split_df(const DevSplitCsr& A, const float4* X, double2* Y, const double2* B, int s, cudaStream_t st) {
-  spmm_df(A, X, OutRows{Y, B, s}, s, st, B != nullptr);  // t = v - A q feeds FP32 local solves: in storage order
+  spmm_df(A, X, OutRows<SpDf<float4>>{Y, B, s}, s, st, B != nullptr);  // t = v - A q feeds FP32 local solves: in storage order
 }
 void spmm_split_df_cols(const DevSplitCsr& A, const float4* X, double2* Y, int s, cudaStream_t st) {
-  spmm_df(A, X, OutCols{Y, A.n}, s, st);
+  spmm_df(A, X, OutCols<SpDf<float4>>{Y, A.n}, s, st);
 }
 void spmm_split_df(const DevSplitCsr& A, const float4* X, float4* Y, int s, cudaStream_t st) {
-  spmm_df(A, X, OutDf{Y, s}, s, st);
+  spmm_df(A, X, OutDf<SpDf<float4>>{Y, s}, s, st);
 }
 void spmm_split_df(const DevSplitCsr& A, const float2* X, double2* Y, int s, cudaStream_t st) {
-  spmm_df(A, X, OutRows{Y, nullptr, s}, s, st);
+  spmm_df(A, X, OutRows<SpDf<float2>>{Y, nullptr, s}, s, st);
 }
 void spmm_split_df(const DevSplitCsr& A, const float2* X, float4* Y, int s, cudaStream_t st, bool ordered) {
-  spmm_df(A, X, OutDf{Y, s}, s, st, ordered);
+  spmm_df(A, X, OutDf<SpDf<float2>>{Y, s}, s, st, ordered);
 }
 
 }  // namespace hz

@@ -5,6 +5,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "f32x2.cuh"
+
 namespace hz {
 
 // Conversions between FP64 and double-float by the IEEE-754 bit layouts, so
@@ -77,16 +79,23 @@ static __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, fl
   sh = t;
 }
 
-// the same with xl = 0
-static __device__ __forceinline__ void df_mac_f(float& sh, float& sl, float ah, float al, float xh) {
-  const float p = __fmul_rn(ah, xh);
-  float e = __fmaf_rn(ah, xh, -p);
-  e = __fmaf_rn(al, xh, e);
-  const float t = __fadd_rn(sh, p);
-  const float z = __fsub_rn(t, sh);
-  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, z)), __fsub_rn(p, z));
-  sl = __fadd_rn(sl, __fadd_rn(err, e));
+// The same on both halves of packed pairs, bit for bit; na = -ah. (The
+// subtractions take p negated: s + p = s - np.)
+static __device__ __forceinline__ void df_add2(pair2& sh, pair2& sl, pair2 np, pair2 e) {
+  const pair2 t = sub2(sh, np);
+  const pair2 z = sub2(t, sh);
+  const pair2 nerr = sub2(add2(np, z), sub2(sh, sub2(t, z)));  // -((sh - (t - z)) + (p - z))
+  sl = add2(sl, sub2(e, nerr));
   sh = t;
+}
+static __device__ __forceinline__ void df_mac2(pair2& sh, pair2& sl, pair2 ah, pair2 na, pair2 al, pair2 xh, pair2 xl) {
+  const pair2 np = mul2(na, xh);
+  df_add2(sh, sl, np, fma2(al, xh, fma2(ah, xl, fma2(ah, xh, np))));
+}
+// xl = 0
+static __device__ __forceinline__ void df_mac2(pair2& sh, pair2& sl, pair2 ah, pair2 na, pair2 al, pair2 xh) {
+  const pair2 np = mul2(na, xh);
+  df_add2(sh, sl, np, fma2(al, xh, fma2(ah, xh, np)));
 }
 
 // (sh, sl) += (h, l)

@@ -104,9 +104,9 @@ __global__ void k_gather(const int* __restrict__ idx, int64_t nrows, const In* _
 // the operand of the product that follows: z in double-float, or in FP32 where z has no more
 __device__ __forceinline__ void put_copy(float4* p, double2 z) {
   const float2 a = df_split(z.x), b = df_split(z.y);
-  *p = make_float4(a.x, a.y, b.x, b.y);
+  *p = make_float4(a.x, b.x, a.y, b.y);
 }
-__device__ __forceinline__ void put_copy(float4* p, float2 z) { *p = make_float4(z.x, 0.f, z.y, 0.f); }
+__device__ __forceinline__ void put_copy(float4* p, float2 z) { *p = make_float4(z.x, z.y, 0.f, 0.f); }
 
 template <typename In, typename Q, typename Out>
 __global__ void k_scatter(const int* __restrict__ own, int64_t n, const In* __restrict__ Xsub, const Q* __restrict__ Qb,

@@ -280,7 +280,7 @@ struct DevKrylov {
 };
 
 // --- double-float products (mixed form, emulated FP64; df.cu) ---
-// X [count] complex FP64 -> (re_hi, re_lo, im_hi, im_lo)
+// X [count] complex FP64 -> (re_hi, im_hi, re_lo, im_lo), the products' operands
 void to_df(const double2* X, float4* Y, int64_t count, cudaStream_t st);
 // Products with A's double-float values; X in double-float, or in FP32 (z of the one-level
 // preconditioner and of the coarse ORAS has no more)

@@ -54,6 +54,7 @@
 #include "kernels.cuh"
 
 #include "cplx.cuh"
+#include "f32x2.cuh"
 
 namespace hz {
 
@@ -158,29 +159,6 @@ struct SweepArgs {
   int s;               // row length of Xsub and Wout (sweep_cols)
   int kids;            // some front of the level has children
 };
-
-// Packed pairs of FP32 numbers: fma.rn.f32x2 rounds each half like a scalar
-// fused multiply-add, and issues half as many instructions.
-using pair2 = unsigned long long;
-__device__ __forceinline__ pair2 pk(float a, float b) {
-  pair2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpk(pair2 p) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p));
-  return r;
-}
-__device__ __forceinline__ pair2 fma2(pair2 a, pair2 b, pair2 c) {
-  pair2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ pair2 add2(pair2 a, pair2 b) {
-  const float2 x = unpk(a), y = unpk(b);
-  return pk(x.x + y.x, x.y + y.y);
-}
 
 // A lane's accumulators, RPT rows x CPT columns
 template <typename V, int S>
