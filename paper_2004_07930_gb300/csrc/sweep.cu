@@ -32,8 +32,8 @@
 // What bounds it: on the 5 Hz workload (0.95M dofs, 64 subdomains, 16
 // columns) the FP32 FMA pipe: 444M factor entries, 114 GFLOP per
 // application, 1.5 ms at the pipe's 74.8 TFLOP/s; with one column HBM: 7.1 GB,
-// 1.05 ms. Measured, whole preconditioner: 4.05 ms (tiles of 64 x 64 per CTA,
-// one output row per thread: 7.16) and 1.69 ms (2.00). The leaf level runs at
+// 1.05 ms. Measured, whole preconditioner: 4.05 ms (tiles of 128 rows,
+// one or a quarter of one per thread: 7.16) and 1.69 ms (2.00). The leaf level runs at
 // 52-55 % of the pipe; the middle levels, 1-10 K small fronts each, spend
 // 30-55 us on the latency of task, indices, inputs and factors in turn.
 //
