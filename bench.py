@@ -443,10 +443,10 @@ MAX_BLOCK = 0
 
 
 def run_spmm_sweep(args):
-    """k_spmm_split alone: for s = 1, 2, 4, 8, 16 the product Y = A X through
+    """k_spmm alone: for s = 1, 2, 4, 8, 16 the product Y = A X through
     hz_apply_A on device blocks, timed by the library's CUDA events around
-    the product only (the layout transposes of hz_apply_A are outside the
-    recorded phase). Algorithmic bytes: 12 per nonzero (value + column),
+    the product only (the input's layout transpose is outside the recorded
+    phase). Algorithmic bytes: 12 per nonzero (value + column),
     row pointers, X and Y once; flops: 4 per nonzero and column."""
     import torch
 
@@ -472,7 +472,7 @@ def run_spmm_sweep(args):
                       "gbs": ph["bytes"] / sec / 1e9, "hbm_frac": ph["bytes"] / sec / 1e9 / hbm,
                       "fp64_gflops": ph["flops"] / sec / 1e9,
                       "fp64_frac": ph["flops"] / sec / 1e9 / FP64_NOMINAL_GFLOPS}
-    print(json.dumps({"mode": "spmm_sweep", "kernel": "k_spmm_split", "config": {"workload": desc},
+    print(json.dumps({"mode": "spmm_sweep", "kernel": "k_spmm", "config": {"workload": desc},
                       "hbm_peak_gbs": hbm, "hbm_peak_kind": peak_kind, "fp64_peak_gflops": FP64_NOMINAL_GFLOPS,
                       "by_block_width": out}), flush=True)
 

@@ -1,7 +1,7 @@
 """Block widths, leaf sizes and restart lengths at the edges of the kernels'
 splits: the front sweeps work on column blocks of 1, 2, 4, 8 and 16 and on
-groups of 16 front rows, the products give a row to 1-8 lanes, the
-Gram-Schmidt products take 32 vectors per launch. Every case against the
+groups of 16 front rows, the products give a row to 1-8 lanes or a thread two
+columns, the Gram-Schmidt products take 12 vectors per launch. Every case against the
 oracle's operators: local solves within 1e-9 (FP64) and 1e-5 (FP32) relative
 L2 and wavefields within 1e-8 at rtol 1e-10, the bounds of the parity tests;
 a product's row of m terms within 2 m eps sum |a x|, eps = 2^-53 (FP64) or
