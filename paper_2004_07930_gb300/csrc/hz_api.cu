@@ -113,6 +113,8 @@ constexpr int MF_TILE_K = 128;     // reduction length per tile (MF_TK in mf.cu)
 // one staging of the input, fewer on levels that would have less than 8 tasks
 // per SM (FP64: 16) otherwise. FP32 keeps four, one for each warp; FP64 goes
 // down to one, whose reduction the warps share. The largest fronts come first.
+// Against always 16 groups: two-level at 5 Hz, 16 columns, 17.6 ms to 18.8; FP64,
+// quarter, 16 columns, 26.4 to 33.5 and the cube, 3 columns, 0.65 to 1.6.
 void level_tasks(bool fwd, bool fp32, const int* list, int count, const std::vector<int>& k, const std::vector<int>& f,
                  const std::vector<int64_t>& rowoff, const std::vector<int64_t>& moff,
                  const std::vector<int64_t>& doff, std::vector<SweepTask>& tasks, int& brows, int& ngroups) {
