@@ -94,6 +94,7 @@ struct MFHost {
   int64_t factor_entries = 0, front_entries = 0;
   std::vector<int> fa_small_ptr, fa_big_ptr, fa_step_ptr, fa_tile_ptr, fi_tile_ptr;  // factorisation schedule
   int max_front = 0, nfronts = 0, nlevels = 0;
+  int task_groups = 0;  // most groups of any sweep task
   std::vector<int> level_ptr;
   std::vector<int> ftask_ptr, btask_ptr, fbrows, bbrows, fgroups, bgroups;  // sweep tasks (DevMF)
   // tensor-core form: tiles and split row blocks per level, levels whose tiles all have at most 64 rows
@@ -107,16 +108,18 @@ constexpr int MF_TILE_ROWS = 128;  // output rows per tile of the tensor-core fo
 constexpr int MF_TILE_K = 128;     // reduction length per tile (MF_TK in mf.cu)
 
 // Sweep tasks of one level (sweep.cu). A task is a run of 16-row groups of
-// one front. Where some reduction of the level is longer than what a CTA keeps
-// in shared memory, a task has at most four groups (one per warp, which
-// follows the input rows as they stream by), elsewhere up to 16, which share
+// one front. Where the input rows stream by (some reduction of the level is
+// longer than what a CTA keeps in shared memory, or `stream`: the persistent
+// form streams every task), a task has at most SW_NW groups, one per warp: the
+// rows pass once, and a warp's second group would need them from the start.
+// Elsewhere up to 16, which share
 // one staging of the input, fewer on levels that would have less than 8 tasks
 // per SM (FP64: 16) otherwise. FP32 keeps four, one for each warp; FP64 goes
 // down to one, whose reduction the warps share. The largest fronts come first.
 // Against always 16 groups: two-level at 5 Hz, 16 columns, 17.6 ms to 18.8; FP64,
 // quarter, 16 columns, 26.4 to 33.5 and the cube, 3 columns, 0.65 to 1.6.
-void level_tasks(bool fwd, bool fp32, const int* list, int count, const std::vector<int>& k, const std::vector<int>& f,
-                 const std::vector<int64_t>& rowoff, const std::vector<int64_t>& moff,
+void level_tasks(bool fwd, bool fp32, bool stream, const int* list, int count, const std::vector<int>& k,
+                 const std::vector<int>& f, const std::vector<int64_t>& rowoff, const std::vector<int64_t>& moff,
                  const std::vector<int64_t>& doff, std::vector<SweepTask>& tasks, int& brows, int& ngroups) {
   int64_t groups = 0;
   std::vector<int> order;
@@ -130,7 +133,8 @@ void level_tasks(bool fwd, bool fp32, const int* list, int count, const std::vec
   brows = 0;
   for (int g : order) brows = std::max(brows, fwd ? k[g] : f[g]);
   const int64_t fill = groups / (fp32 ? 1216 : 2432);
-  const int most = (int)std::min<int64_t>(std::max<int64_t>(fill, fp32 ? 4 : 1), brows > MF_RES ? 4 : 16);
+  const int most = (int)std::min<int64_t>(std::max<int64_t>(fill, fp32 ? SW_NW : 1),
+                                          stream || brows > MF_RES ? SW_NW : 16);
   for (int g : order) {
     const int nout = fwd ? f[g] : k[g];
     const int ng = (nout + MF_GR - 1) / MF_GR;
@@ -285,11 +289,13 @@ void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const Fron
   for (int l = 0; l <= maxh; ++l) {
     const int* list = level_list.data() + info.level_ptr[l];
     const int count = info.level_ptr[l + 1] - info.level_ptr[l];
-    level_tasks(true, fp32, list, count, k, f, rowoff, Moff, Doff, ftasks, info.fbrows[l], info.fgroups[l]);
-    level_tasks(false, fp32, list, count, k, f, rowoff, MToff, Doff, btasks, info.bbrows[l], info.bgroups[l]);
+    level_tasks(true, fp32, persistent, list, count, k, f, rowoff, Moff, Doff, ftasks, info.fbrows[l], info.fgroups[l]);
+    level_tasks(false, fp32, persistent, list, count, k, f, rowoff, MToff, Doff, btasks, info.bbrows[l], info.bgroups[l]);
     info.ftask_ptr.push_back((int)ftasks.size());
     info.btask_ptr.push_back((int)btasks.size());
   }
+  for (const std::vector<SweepTask>* v : {&ftasks, &btasks})
+    for (const SweepTask& t : *v) info.task_groups = std::max<int>(info.task_groups, t.ng);
   // tensor-core form: tiles (front, first output row, first reduction index, partial slot) and row
   // blocks (front, first output row, tiles, first slot); slots restart at 0 on every level. A row block
   // covered by a single tile finishes inside the tile (slot -1); the others sum their partial tiles in
@@ -371,7 +377,8 @@ void build_mf(const std::vector<const CsrC*>& mats, const std::vector<const Fron
   mf.btasks = pool.upload(btasks, st);
   mf.csrc = pool.upload(csrc, st);
   if (persistent) {
-    // the same tasks, the backward ones from the roots down. Forward: a front waits for its children
+    // the same tasks (no more groups than warps: every one of them streams), the backward ones from the
+    // roots down. Forward: a front waits for its children
     // that have rows (a child without rows has no update rows either and contributes nothing);
     // backward: a front waits for its nearest ancestor with pivots, which finishes only after all of
     // its own ancestors
@@ -2519,3 +2526,25 @@ extern "C" int hz_fwi_gradient(hz_ctx* c, const double* src_xyz, const double* s
     return rc;
   });
 }
+
+// Entries for the tests of the sweeps' task rule (not part of the public ABI).
+// Tasks of one level of n fronts (pivots k, orders f): (front, first group,
+// groups) triples to out, at most cap of them; returns their number, the
+// longest reduction to *rows.
+extern "C" int hz_internal_level_tasks(int fwd, int fp32, int stream, int n, const int* k, const int* f, int* out,
+                                       int cap, int* rows) {
+  std::vector<int> list(n), kv(k, k + n), fv(f, f + n);
+  for (int g = 0; g < n; ++g) list[g] = g;
+  const std::vector<int64_t> zero(n, 0);
+  std::vector<SweepTask> tasks;
+  int groups = 0;
+  level_tasks(fwd != 0, fp32 != 0, stream != 0, list.data(), n, kv, fv, zero, zero, zero, tasks, *rows, groups);
+  for (size_t t = 0; t < tasks.size() && (int)t < cap; ++t) {
+    out[3 * t] = tasks[t].front;
+    out[3 * t + 1] = tasks[t].g0;
+    out[3 * t + 2] = tasks[t].ng;
+  }
+  return (int)tasks.size();
+}
+// Most groups of any sweep task of the fine level
+extern "C" int hz_internal_task_groups(const hz_ctx* c) { return c ? c->lf.info.task_groups : -1; }

@@ -38,6 +38,7 @@ struct DevSplitCsr {
 // bytes, (re, re, im, im), the operand pairs of the packed FP32 multiply-add.
 constexpr int MF_GR = 16;      // rows per group
 constexpr int MF_CHUNK = 128;  // reduction indices summed before the running total takes them
+constexpr int SW_NW = 4;       // warps of a sweep CTA, one group each at a time
 constexpr int MF_RES = 256;    // longest reduction whose input rows a sweep task keeps in shared memory
 __host__ __device__ inline int mf_group_rows(int nout, int g) {  // padded rows of group g of nout rows
   const int nr = nout - MF_GR * g;

@@ -60,7 +60,6 @@ namespace hz {
 
 namespace {
 
-constexpr int SW_NW = 4;  // warps per CTA
 constexpr int SW_THREADS = 32 * SW_NW;
 constexpr int SW_NST = 2;  // ring stages per warp
 
