@@ -647,6 +647,208 @@ __global__ void __launch_bounds__(SW_THREADS, sw_min_blocks<V, S, FWD, STREAM>()
 }
 
 // ---------------------------------------------------------------------------
+// One column in complex FP32, long reductions on a level of few groups: what
+// counts is the chain of one row, its staged inputs, ring stages and
+// multiply-adds in turn. A CTA takes one group, and its warps one chunk
+// (MF_CHUNK reduction indices) each at a time; the chunks' sums meet in shared
+// memory and are added in order, the order of the sums of the other forms.
+// Against k_sweep_level, whose warps follow their group from end to end
+// (quarter workload, one column, us a level): 109 tasks 39 -> 20, 193 30 -> 17,
+// 264 35 -> 29, 480 24 -> 21, but 686 20 -> 22 and 1161 23 -> 36, where the
+// level is wide enough and a CTA that stages its input for one group reads
+// more; hence up to LG_TASKS, four CTAs of the wider form per SM. The
+// application: 0.81 -> 0.60 ms (the earlier tiles, split at 128 indices: 0.67);
+// 5 Hz workload 1.68 -> 1.66. Two ring stages: three and four take the CTAs
+// their shared memory (0.61 -> 0.65 with every such level in this form).
+// ---------------------------------------------------------------------------
+constexpr int LG_KC = 32;                       // indices per ring stage (4 KB)
+constexpr int LG_NST = 2;                       // ring stages per warp
+constexpr unsigned LG_TASKS = 608;
+constexpr int LG_STAGE = LG_KC * MF_GR;         // entries per stage
+constexpr int LG_ROWS = SW_NW * MF_CHUNK;       // input rows of a window, one chunk per warp
+constexpr int LG_RPT = LG_ROWS / SW_THREADS;    // rows per thread
+constexpr size_t LG_SMEM = (size_t)SW_NW * LG_NST * LG_STAGE * sizeof(float2) + 2 * LG_ROWS * sizeof(float2) +
+                           2 * SW_NW * MF_GR * sizeof(float2);
+
+// group g of the task; `wait` as in sweep_task_t
+template <bool FWD, typename Wait>
+__device__ __forceinline__ bool sweep_long(const SweepArgs<float2>& A, const SweepTask& T, int g, unsigned char* smem,
+                                           Wait&& wait) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int k = T.k, f = T.f, nout = FWD ? f : k;
+  const int lo = FWD ? 0 : MF_GR * g, hi = FWD ? min(k, MF_GR * (g + 1)) : f;
+  const int c0 = lo / MF_CHUNK, cend = (hi + MF_CHUNK - 1) / MF_CHUNK;  // the group's chunks
+  const int nrp = mf_group_rows(nout, g), r = MF_GR * g + tid;        // threads below MF_GR: an output row each
+  float2* const ring = reinterpret_cast<float2*>(smem) + (size_t)warp * LG_NST * LG_STAGE;
+  float2* const bs = reinterpret_cast<float2*>(smem) + (size_t)SW_NW * LG_NST * LG_STAGE;  // [2][LG_ROWS]
+  float2* const parts = bs + 2 * LG_ROWS;                                                  // [2][warp][row]
+  float2* const own = A.Wout + T.row;
+  const float2* const M = A.M + T.m + (FWD ? mf_fwd_before(k, g) : mf_bwd_before(f, g));
+
+  // ring: the stages of the warp's chunks c0 + warp, + SW_NW, ... in order; none spans two chunks
+  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+  int ic = c0 + warp, il = max(lo, ic * MF_CHUNK), islot = 0;
+  auto issue = [&]() {
+    if (ic < cend) {
+      const int end = min(hi, (ic + 1) * MF_CHUNK), n = min(LG_KC, end - il), bytes = n * nrp * (int)sizeof(float2);
+      const char* src = reinterpret_cast<const char*>(M + (int64_t)(il - lo) * nrp) + lane * 16;
+      const uint32_t dst = ring_s + islot * (LG_STAGE * (int)sizeof(float2)) + lane * 16;
+#pragma unroll
+      for (int o = 0; o < LG_STAGE * (int)sizeof(float2); o += 512)
+        if (o + lane * 16 < bytes) cp_async16(dst + o, src + o);
+      il += n;
+      if (il == end) {
+        ic += SW_NW;
+        il = ic * MF_CHUNK;
+      }
+    }
+    cp_async_commit();
+    islot = islot + 1 == LG_NST ? 0 : islot + 1;
+  };
+#pragma unroll
+  for (int i = 0; i < LG_NST - 1; ++i) issue();
+
+  // input rows of the window from chunk cw on: their sources, then their values
+  int xr[LG_RPT];
+  int2 cc[LG_RPT];
+  float2 v[LG_RPT], w0[LG_RPT], w1[LG_RPT];
+  auto load_idx = [&](int cw) {
+#pragma unroll
+    for (int i = 0; i < LG_RPT; ++i) {
+      const int l = cw * MF_CHUNK + i * SW_THREADS + tid;
+      xr[i] = -1;
+      cc[i] = make_int2(-1, -1);
+      if (l >= lo && l < hi) {
+        if (FWD || l >= k) xr[i] = __ldg(A.rows + T.row + l);
+        if (FWD && A.kids) cc[i] = __ldg(A.csrc + T.row + l);
+      }
+    }
+  };
+  auto load_val = [&](int cw) {
+#pragma unroll
+    for (int i = 0; i < LG_RPT; ++i) {
+      const int l = cw * MF_CHUNK + i * SW_THREADS + tid;
+      v[i] = w0[i] = w1[i] = make_float2(0.f, 0.f);
+      if (l >= lo && l < hi) {
+        v[i] = __ldcg(FWD || xr[i] >= 0 ? A.Xsub + xr[i] : own + l);
+        if (cc[i].x >= 0) w0[i] = __ldcg(A.Wout + cc[i].x);
+        if (cc[i].y >= 0) w1[i] = __ldcg(A.Wout + cc[i].y);
+      }
+    }
+  };
+  auto store_val = [&](float2* b) {
+#pragma unroll
+    for (int i = 0; i < LG_RPT; ++i)
+      b[i * SW_THREADS + tid] = FWD && A.kids ? c_add(c_add(v[i], w0[i]), w1[i]) : v[i];
+  };
+  load_idx(c0);
+  int xo = 0;
+  int2 ce = make_int2(-1, -1);
+  float2 di = make_float2(0.f, 0.f), tot = di;
+  const bool out = tid < MF_GR && r < nout;
+  if (out) {
+    if (!FWD) xo = __ldg(A.rows + T.row + r);
+    if (FWD && A.kids && r >= k) ce = __ldg(A.csrc + T.row + r);
+    if (FWD && r < k) di = __ldg(A.Dinv + T.d + r);
+  }
+  if (!wait()) return false;
+
+  load_val(c0);
+  if (c0 + SW_NW < cend) load_idx(c0 + SW_NW);
+  store_val(bs);
+  auto add_parts = [&](int cw, int buf) {  // chunks cw..cw + 3, in order
+    if (tid < MF_GR)
+      for (int w = 0; w < SW_NW && cw + w < cend; ++w) {
+        const float2 q = parts[(buf * SW_NW + w) * MF_GR + tid];
+        tot = cw + w == c0 ? q : c_add(tot, q);
+      }
+  };
+  int slot = 0, buf = 0;
+  for (int cw = c0; cw < cend; cw += SW_NW, buf ^= 1) {
+    __syncthreads();
+    const bool more = cw + SW_NW < cend;
+    if (more) {
+      load_val(cw + SW_NW);
+      if (cw + 2 * SW_NW < cend) load_idx(cw + 2 * SW_NW);
+    }
+    if (cw > c0) add_parts(cw - SW_NW, buf ^ 1);
+    if (cw + warp < cend) {
+      const int p = min(lane & 7, nrp / 2 - 1), end = min(hi, (cw + warp + 1) * MF_CHUNK);
+      int ck = max(lo, (cw + warp) * MF_CHUNK);
+      pair2 re = 0, im = 0;
+      while (ck < end) {
+        cp_async_wait<LG_NST - 2>();
+        __syncwarp();
+        issue();
+        const int n = min(LG_KC, end - ck);
+        const float4* a = reinterpret_cast<const float4*>(ring + slot * LG_STAGE) + p;
+        const float2* b = bs + buf * LG_ROWS + (ck - cw * MF_CHUNK);
+        auto step = [&](const float4 t, const float2 bv) {
+          const pair2 ar = pk(t.x, t.y), ai = pk(t.z, t.w);
+          const pair2 br = pk(bv.x, bv.x), bi = pk(bv.y, bv.y), nbi = pk(-bv.y, -bv.y);
+          re = fma2(ar, br, fma2(ai, nbi, re));
+          im = fma2(ar, bi, fma2(ai, br, im));
+        };
+        int kk = 0;
+#pragma unroll 1
+        for (; kk + 8 <= n; kk += 8) {
+          float4 t[8];
+          float2 bv[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            t[u] = a[(kk + u) * (nrp / 2)];
+            bv[u] = b[kk + u];
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) step(t[u], bv[u]);
+        }
+#pragma unroll 1
+        for (; kk < n; ++kk) step(a[kk * (nrp / 2)], b[kk]);
+        ck += n;
+        slot = slot + 1 == LG_NST ? 0 : slot + 1;
+      }
+      const float2 x = unpk(re), y = unpk(im);
+      if (lane < nrp / 2)
+        reinterpret_cast<float4*>(parts)[((buf * SW_NW + warp) * MF_GR) / 2 + lane] = make_float4(x.x, y.x, x.y, y.y);
+    }
+    if (more) store_val(bs + (buf ^ 1) * LG_ROWS);
+  }
+  __syncthreads();
+  if (cend > c0) {
+    const int nw = (cend - c0 + SW_NW - 1) / SW_NW;
+    add_parts(c0 + (nw - 1) * SW_NW, (nw - 1) & 1);
+  }
+  if (out) {
+    if (!FWD) {
+      A.Xsub[xo] = tot;
+    } else {
+      float2 x0 = make_float2(0.f, 0.f), x1 = x0;
+      if (ce.x >= 0) x0 = __ldcg(A.Wout + ce.x);
+      if (ce.y >= 0) x1 = __ldcg(A.Wout + ce.y);
+      if (r < k) tot = cend > 1 ? mul_dinv<true>(tot, di) : mul_dinv<false>(tot, di);
+      if (ce.x >= 0) tot = c_add(tot, x0);
+      if (ce.y >= 0) tot = c_add(tot, x1);
+      own[r] = tot;
+    }
+  }
+  return true;
+}
+
+// One level of one sweep in that form: blockIdx = task * SW_NW + group of the task.
+template <bool FWD>
+__global__ void __launch_bounds__(SW_THREADS, 5) k_sweep_long(SweepArgs<float2> A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_trigger();
+  const SweepTask T = A.tasks[blockIdx.x / SW_NW];
+  const int q = blockIdx.x % SW_NW;
+  if (q >= T.ng) return;  // the task's first CTA waits for the previous launch
+  sweep_long<FWD>(A, T, T.g0 + q, smem_raw, [] {
+    pdl_wait();
+    return true;
+  });
+}
+
+// ---------------------------------------------------------------------------
 // Persistent sweeps (option persistent_sweeps): one launch per direction over
 // every level. Resident CTAs take the tasks in level order through a ticket
 // counter (the forward sweep from the leaves up, the backward sweep from the
@@ -736,6 +938,11 @@ void launch_level(const DevMF& mf, SweepArgs<V>& A, int l, cudaStream_t st) {
   const int ncb = A.s / S, rows = (FWD ? mf.fbrows_h : mf.bbrows_h)[l];
   const unsigned grid = (unsigned)(ptr[l + 1] - ptr[l]) * ncb;
   A.tasks = (FWD ? mf.ftasks : mf.btasks) + ptr[l];
+  if constexpr (sizeof(V) == 8 && S == 1)
+    if (rows > MF_RES && grid < LG_TASKS) {
+      launch_k(true, k_sweep_long<FWD>, grid * SW_NW, SW_THREADS, LG_SMEM, st, A);
+      return;
+    }
   if (rows <= MF_RES)
     launch_k(true, k_sweep_level<V, S, FWD, false>, grid, SW_THREADS, sw_smem<V, S, FWD, false>(rows), st, A, ncb);
   else
@@ -821,6 +1028,8 @@ void attrs_sf() {
   cudaFuncSetAttribute(k_sweep_level<V, S, FWD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, whole);
   cudaFuncSetAttribute(k_sweep_level<V, S, FWD, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, stream);
   cudaFuncSetAttribute(k_sweep_all<V, S, FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, stream);
+  if constexpr (sizeof(V) == 8 && S == 1)
+    cudaFuncSetAttribute(k_sweep_long<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LG_SMEM);
 }
 template <typename V, int S>
 void attrs_s() {
