@@ -966,18 +966,18 @@ void apply_oras(LevelDev& L, const double2* V, double2* Zout, const double2* Qad
   const double fflops = 8.0 * s * 2.0 * L.info.factor_entries;
   int p0 = prof ? prof->begin(PH_RESTRICT, st) : -1;
   if (L.mf.fp32)
-    gather_rows(L.mf.gidx, L.sub_rows, V, (float2*)Xsub, s, st);
+    gather_rows(L.mf, V, (float2*)Xsub, s, st);
   else
-    gather_rows(L.mf.gidx, L.sub_rows, V, Xsub, s, st);
+    gather_rows(L.mf, V, Xsub, s, st);
   if (prof) prof->end(p0, st, 0.0, 0.0);
   int p1 = prof ? prof->begin(PH_FRONTS, st) : -1;
   run_graph(graph, s, st, [&]() { mf_solve(L.mf, Xsub, s, st); });
   if (prof) prof->end(p1, st, fflops, fbytes);
   int p2 = prof ? prof->begin(PH_RESTRICT, st) : -1;
   if (L.mf.fp32)
-    scatter_owned(L.mf.own, L.n, (const float2*)Xsub, Qadd, Zout, s, st, Zdf, Zf);
+    scatter_owned(L.mf, L.n, (const float2*)Xsub, Qadd, Zout, s, st, Zdf, Zf);
   else
-    scatter_owned(L.mf.own, L.n, Xsub, Qadd, Zout, s, st);
+    scatter_owned(L.mf, L.n, Xsub, Qadd, Zout, s, st);
   if (prof) prof->end(p2, st, 0.0, rbytes);
 }
 
@@ -1003,9 +1003,9 @@ void coarse_solve(hz_ctx* c, const double2* rH, double2* yH, int s) {
     CK(cudaMemsetAsync(c->yH32, 0, vs * sizeof(float2), st));
     krylov_start(K, c->rH32, st);
     for (int j = 0; j < K.m; ++j) {
-      gather_rows(L.mf.gidx, L.sub_rows, V + j * vs, Xs, s, st);
+      gather_rows(L.mf, V + j * vs, Xs, s, st);
       mf_solve(L.mf, Xs, s, st);
-      scatter_owned(L.mf.own, L.n, Xs, (const float2*)nullptr, Zk + j * vs, s, st);
+      scatter_owned(L.mf, L.n, Xs, (const float2*)nullptr, Zk + j * vs, s, st);
       spmm_split_f32(c->E, Zk + j * vs, (float2*)K.W, s, st);
       krylov_arnoldi(K, j, st);
     }
@@ -1135,14 +1135,14 @@ void apply_prec(hz_ctx* c, const double2* V, double2* Zout, int s) {
                 6.0 * (c->A.nnz_re + c->A.nnz_im) + 16.0 * (n + 1) + 24.0 * n * s);
     LevelDev& L = c->lf;
     int p0 = c->prof.begin(PH_RESTRICT, st);
-    gather_rows(L.mf.gidx, L.sub_rows, c->t32, (float2*)c->Xsub, s, st);
+    gather_rows(L.mf, c->t32, (float2*)c->Xsub, s, st);
     c->prof.end(p0, st, 0.0, 0.0);
     int p1 = c->prof.begin(PH_FRONTS, st);
     run_graph(gf, s, st, [&]() { mf_solve(L.mf, c->Xsub, s, st); });
     c->prof.end(p1, st, 8.0 * s * 2.0 * L.info.factor_entries,
                 8.0 * 2.0 * L.info.factor_entries + 2.0 * 8.0 * s * L.sub_rows);
     int p2 = c->prof.begin(PH_RESTRICT, st);
-    scatter_owned(L.mf.own, L.n, (const float2*)c->Xsub, c->q32, Zout, s, st, c->df ? c->Xdf : nullptr);  // z = M1^{-1} t + q
+    scatter_owned(L.mf, L.n, (const float2*)c->Xsub, c->q32, Zout, s, st, c->df ? c->Xdf : nullptr);  // z = M1^{-1} t + q
     c->prof.end(p2, st, 0.0, 4.0 * L.sub_rows + 16.0 * L.sub_rows * s + 4.0 * L.n + 32.0 * L.n * s);
     return;
   }

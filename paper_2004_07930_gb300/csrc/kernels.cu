@@ -129,43 +129,44 @@ __global__ void k_scatter(const int* __restrict__ own, int64_t n, const In* __re
 }
 
 template <typename In, typename Out>
-static void gather_t(const int* idx, int64_t nrows, const In* X, Out* Y, int s, cudaStream_t st) {
+static void gather_t(const DevMF& mf, const In* X, Out* Y, int s, cudaStream_t st) {
+  const int64_t nrows = mf.nsub_rows;
   if (nrows * s == 0) return;
-  const int cols = sweep_cols(s);
+  const int cols = sub_cols(mf, s);
   const dim3 b(cols, std::max(1, 256 / cols));
-  { k_gather<<<grid_for(nrows, b.y), b, 0, st>>>(idx, nrows, X, Y, s, cols); count_launch(); }
+  { k_gather<<<grid_for(nrows, b.y), b, 0, st>>>(mf.gidx, nrows, X, Y, s, cols); count_launch(); }
 }
 template <typename In, typename Q, typename Out>
-static void scatter_t(const int* own, int64_t n, const In* Xsub, const Q* Qb, Out* Z, int s, cudaStream_t st,
+static void scatter_t(const DevMF& mf, int64_t n, const In* Xsub, const Q* Qb, Out* Z, int s, cudaStream_t st,
                       float4* Zdf = nullptr, float2* Zf = nullptr) {
   if (n * s == 0) return;
   const dim3 b(s, std::max(1, 256 / s));
-  { k_scatter<<<grid_for(n, b.y), b, 0, st>>>(own, n, Xsub, Qb, Z, s, sweep_cols(s), Zdf, Zf); count_launch(); }
+  { k_scatter<<<grid_for(n, b.y), b, 0, st>>>(mf.own, n, Xsub, Qb, Z, s, sub_cols(mf, s), Zdf, Zf); count_launch(); }
 }
 
-void gather_rows(const int* idx, int64_t nrows, const double2* X, double2* Y, int s, cudaStream_t st) {
-  gather_t(idx, nrows, X, Y, s, st);
+void gather_rows(const DevMF& mf, const double2* X, double2* Y, int s, cudaStream_t st) {
+  gather_t(mf, X, Y, s, st);
 }
-void gather_rows(const int* idx, int64_t nrows, const double2* X, float2* Y, int s, cudaStream_t st) {
-  gather_t(idx, nrows, X, Y, s, st);
+void gather_rows(const DevMF& mf, const double2* X, float2* Y, int s, cudaStream_t st) {
+  gather_t(mf, X, Y, s, st);
 }
-void gather_rows(const int* idx, int64_t nrows, const float2* X, float2* Y, int s, cudaStream_t st) {
-  gather_t(idx, nrows, X, Y, s, st);
+void gather_rows(const DevMF& mf, const float2* X, float2* Y, int s, cudaStream_t st) {
+  gather_t(mf, X, Y, s, st);
 }
-void scatter_owned(const int* own, int64_t n, const double2* Xsub, const double2* Q, double2* Z, int s,
+void scatter_owned(const DevMF& mf, int64_t n, const double2* Xsub, const double2* Q, double2* Z, int s,
                    cudaStream_t st) {
-  scatter_t(own, n, Xsub, Q, Z, s, st);
+  scatter_t(mf, n, Xsub, Q, Z, s, st);
 }
-void scatter_owned(const int* own, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
+void scatter_owned(const DevMF& mf, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
                    cudaStream_t st, float4* Zdf, float2* Zf) {
-  scatter_t(own, n, Xsub, Q, Z, s, st, Zdf, Zf);
+  scatter_t(mf, n, Xsub, Q, Z, s, st, Zdf, Zf);
 }
-void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
+void scatter_owned(const DevMF& mf, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
                    cudaStream_t st, float4* Zdf) {
-  scatter_t(own, n, Xsub, Q, Z, s, st, Zdf);
+  scatter_t(mf, n, Xsub, Q, Z, s, st, Zdf);
 }
-void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st) {
-  scatter_t(own, n, Xsub, Q, Z, s, st);
+void scatter_owned(const DevMF& mf, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st) {
+  scatter_t(mf, n, Xsub, Q, Z, s, st);
 }
 
 __global__ void k_zero(double2* X, int64_t count) {

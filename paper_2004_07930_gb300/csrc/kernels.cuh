@@ -224,25 +224,26 @@ void spmm_real(int64_t nrows, const int64_t* rp, const int32_t* col, const doubl
                double2* Y, int s, cudaStream_t st);
 
 // --- restriction / prolongation ---
-// Sub-vectors have rows of sweep_cols(s) entries, the columns past s zero.
-int sweep_cols(int s);  // sweep.cu
-// Y[r][:] = X[idx[r]][:] (R_i), in the sub-vector's precision
-void gather_rows(const int* idx, int64_t nrows, const double2* X, double2* Y, int s, cudaStream_t st);
-void gather_rows(const int* idx, int64_t nrows, const double2* X, float2* Y, int s, cudaStream_t st);
-void gather_rows(const int* idx, int64_t nrows, const float2* X, float2* Y, int s, cudaStream_t st);
+// Sub-vectors have rows of sub_cols(mf, s) entries, the columns past s zero.
+int sweep_cols(int s);                    // sweep.cu
+int sub_cols(const DevMF& mf, int s);     // mf.cu
+// Y[r][:] = X[gidx[r]][:] (R_i), in the sub-vector's precision
+void gather_rows(const DevMF& mf, const double2* X, double2* Y, int s, cudaStream_t st);
+void gather_rows(const DevMF& mf, const double2* X, float2* Y, int s, cudaStream_t st);
+void gather_rows(const DevMF& mf, const float2* X, float2* Y, int s, cudaStream_t st);
 // Z[r][:] = Xsub[own[r]][:] (+ Q[r][:]), in Z's precision (Q may be NULL); Zdf: Z in double-float beside it,
 // Zf: the FP32 sub-vector values themselves (Z without Q)
-void scatter_owned(const int* own, int64_t n, const double2* Xsub, const double2* Q, double2* Z, int s,
+void scatter_owned(const DevMF& mf, int64_t n, const double2* Xsub, const double2* Q, double2* Z, int s,
                    cudaStream_t st);
-void scatter_owned(const int* own, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
+void scatter_owned(const DevMF& mf, int64_t n, const float2* Xsub, const double2* Q, double2* Z, int s,
                    cudaStream_t st, float4* Zdf = nullptr, float2* Zf = nullptr);
-void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
+void scatter_owned(const DevMF& mf, int64_t n, const float2* Xsub, const float2* Q, double2* Z, int s,
                    cudaStream_t st, float4* Zdf = nullptr);
-void scatter_owned(const int* own, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st);
+void scatter_owned(const DevMF& mf, int64_t n, const float2* Xsub, const float2* Q, float2* Z, int s, cudaStream_t st);
 
 // --- multifrontal ---
 void mf_factor(DevMF& mf, double tau_abs, cudaStream_t st);
-void mf_solve(DevMF& mf, void* Xsub, int s, cudaStream_t st);  // Xsub double2 or float2 (mf.fp32), [rows][sweep_cols(s)]
+void mf_solve(DevMF& mf, void* Xsub, int s, cudaStream_t st);  // Xsub double2 or float2 (mf.fp32), [rows][sub_cols(mf, s)]
 void sweep_attrs(bool fp32);                                         // sweep.cu
 void sweep_solve(DevMF& mf, void* Xsub, int cols, cudaStream_t st);  // sweep.cu; cols = sweep_cols(s)
 bool mf_tc_usable(const DevMF& mf, int s);  // the block width runs the tensor-core sweeps
