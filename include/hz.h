@@ -288,8 +288,13 @@ typedef struct hz_server hz_server;
 int hz_server_create(hz_ctx* ctx, int32_t slots, hz_server** out);
 /* Device bytes one slot (right-hand-side column) of a server on ctx costs:
  * the server's blocks plus the context workspace of one column (Krylov basis,
- * preconditioner blocks, local sub-vectors of both levels). A caller admits by
- * device footprint by creating servers with budget / column_bytes slots. */
+ * preconditioner blocks, local sub-vectors of both levels). The sub-vectors
+ * come in whole column blocks, so the figure holds for servers of 1, 2, 4, 8,
+ * 16 or a multiple of 8 slots, and one of any other number costs up to as
+ * much as the next of these. A caller admits by device footprint by creating
+ * servers with budget / column_bytes slots, rounded down to one of these
+ * numbers; each server holds one more column of n complex numbers to stage a
+ * request. */
 int hz_server_column_bytes(const hz_ctx* ctx, double* bytes);
 int hz_server_submit(hz_server* srv, int64_t request_id, const double* src_xyz, const double* src_amp, int32_t ns);
 int hz_server_step(hz_server* srv, int64_t* done_ids, int32_t cap, int32_t* ndone);

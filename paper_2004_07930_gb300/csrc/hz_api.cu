@@ -794,13 +794,15 @@ struct hz_ctx {
 
 namespace {
 
+constexpr int KRYLOV_CTAS = 304;  // CTAs of the Gram-Schmidt products, two per SM
+
 void alloc_krylov(DevKrylov& K, int64_t n, int s, int m, DevPool& p, cudaStream_t st, bool fp32, bool df = false) {
   K.n = n;
   K.s = s;
   K.m = m;
   K.fp32 = fp32 ? 1 : 0;
   K.df = (df && !fp32) ? 1 : 0;
-  K.nblk = 304;
+  K.nblk = KRYLOV_CTAS;
   if (K.df) {
     K.Wdf = p.alloc<float4>((size_t)n * s);
     K.hdf = p.alloc<float4>((size_t)(m + 1) * s);
@@ -880,7 +882,7 @@ void ensure_workspace(hz_ctx* c, int s) {
     B.m = m;
     B.s = s;
     B.n = n;
-    B.nblk = 304;
+    B.nblk = KRYLOV_CTAS;
     B.V = (double2*)c->Kout.V;
     B.Zk = (double2*)c->Kout.Zk;
     B.W = (double2*)c->Kout.W;
@@ -2125,26 +2127,51 @@ struct hz_server {
   };
 };
 
-// Device bytes that one right-hand-side column adds to a server on this
-// context: the server's own B, X, R columns plus the context workspace of
-// one column (the blocks of M^{-1} and of the outer Krylov basis, the local
-// sub-vectors and front vectors of both levels, the inner coarse Krylov
-// basis), as ensure_workspace allocates them.
+// Device bytes of one column of a Krylov space (alloc_krylov) of n rows,
+// restart length m and es bytes per entry
+static double krylov_column_bytes(double n, double m, double es, bool df) {
+  double b = es * n * (2.0 * m + 2.0);                            // V, Zk, W
+  if (df) b += 16.0 * (n + m + 1);                                // W and the coefficients in double-float
+  b += 16.0 * ((m + 1) * m + KRYLOV_CTAS * (m + 2));              // H, partial products
+  return b + 16.0 * (3.0 * (m + 1) + 2.0 * m) + 8.0 * m + 40.0;   // h1, h2, g, sn, y, cs, per-column scalars
+}
+
+// Device bytes of one slot of a server on this context: its B, X, R columns
+// plus the context workspace of one column, as ensure_workspace allocates
+// them. The sub-vectors and front vectors have rows of sweep_cols(slots)
+// entries, so that this is exact where the slots are whole column blocks
+// (sweep_cols(slots) == slots), and a server of any other number holds no more
+// than one of the next such number. No single figure would do for every
+// number of slots: 9 slots hold 16 columns of those vectors, 5 % of the column
+// on the 5 Hz workload in the mixed form, which a server of 32 does not need.
+// What grows with the square of the block (block_arnoldi) or has a fixed part
+// (recycle) is counted at its largest share.
 static double column_bytes(const hz_ctx* c) {
-  const double n = (double)c->space.n, m = c->opt.restart;
+  const double n = (double)c->space.n, m = c->opt.restart, s = c->opt.max_block;
   const double ef = c->lf.mf.fp32 ? 8.0 : 16.0;
+  auto local = [&](const LevelDev& L) {
+    const double tiles = L.mf.tc ? (double)L.mf.max_slots * MF_TILE_ROWS : 0.0;
+    return (double)L.sub_rows + (double)L.mf.rows_total + tiles;
+  };
   double b = 3.0 * 16.0 * n;                                    // server B, X, R
   b += 6.0 * 16.0 * n;                                          // context B, X, R, T, Q, U
-  b += ef * ((double)c->lf.sub_rows + (double)c->lf.mf.rows_total + (double)c->lf.mf.max_slots * MF_TILE_ROWS);
-  b += 16.0 * n * (2.0 * m + 2.0);                              // V, Zk, W
-  if (c->df) b += 16.0 * n * 2.0;                               // double-float W and product input
+  b += ef * local(c->lf);
+  b += krylov_column_bytes(n, m, 16.0, c->df && !c->opt.block_arnoldi && c->opt.recycle == 0);
+  b += 16.0;                                                    // norms
+  if (c->df) b += 16.0 * n;                                     // the product's operand
+  if (c->opt.recycle > 0) {
+    const double rk = c->opt.recycle;
+    b += 16.0 * ((m + 1) * m + m * rk + rk * rk * (1.0 + KRYLOV_CTAS));
+  }
+  if (c->opt.block_arnoldi)
+    b += 16.0 * s * ((m + 1) * m + (m + 1) + m + (KRYLOV_CTAS + 2.0) * (m + 1) + 3.0 + m) + 8.0 * s * m + 8.0;
   if (c->has_coarse) {
     const double nh = (double)c->cspace.n, ec = c->lc.mf.fp32 ? 8.0 : 16.0, ek = c->coarse32 ? 8.0 : 16.0;
-    const double mi = std::max(1, c->opt.coarse_inner_its);
     b += 2.0 * 16.0 * nh;                                       // r_H, y_H
-    b += ec * ((double)c->lc.sub_rows + (double)c->lc.mf.rows_total + (double)c->lc.mf.max_slots * MF_TILE_ROWS);
-    if (c->opt.coarse_mode == HZ_COARSE_GMRES) b += ek * nh * (2.0 * mi + 2.0);
-    if (c->df && !c->coarse32 && c->opt.coarse_mode == HZ_COARSE_GMRES) b += 16.0 * nh * 2.0;
+    b += ec * local(c->lc);
+    if (c->opt.coarse_mode == HZ_COARSE_GMRES)
+      b += krylov_column_bytes(nh, std::max(1, c->opt.coarse_inner_its), ek, c->df && !c->coarse32);
+    if (c->df && !c->coarse32) b += 16.0 * nh;
     if (c->coarse32) b += 8.0 * (2.0 * nh + 3.0 * n);
   }
   return b;

@@ -28,8 +28,9 @@ from . import hz
 def slots_for_budget(solvers, device_budget, max_slots=64):
     """Slots per frequency: an equal share of `device_budget` bytes divided by
     the bytes of one column on that frequency's solver, rounded down to a
-    power of two (the kernels run the instantiation for the next power of two
-    of the block width, so other widths pay for idle columns), at least 1."""
+    power of two (the front sweeps and their vectors come in whole column
+    blocks, and the figure holds for those: 9 slots would hold and compute 16
+    columns), at least 1."""
     share = float(device_budget) / len(solvers)
     out = {}
     for f, S in solvers.items():
