@@ -76,16 +76,16 @@ struct OutDf {  // Y = A X in double-float, renormalised, (re hi, re lo, im hi, 
     Y[r * s + c] = y;
   }
 };
-template <typename XT, typename Out>
-void spmm_df(const DevSplitCsr& A, const XT* X, Out out, int s, cudaStream_t st, bool ordered = false) {
-  spmm_launch<SpDf<XT>>(A.n, s, A.rp_re, A.col_re, A.val_re_df, A.rp_im, A.col_im, A.val_im_df, X, out, st, ordered);
+template <bool ORDERED, typename XT, typename Out>
+void spmm_df(const DevSplitCsr& A, const XT* X, Out out, int s, cudaStream_t st) {
+  spmm_launch<SpDf<XT>, ORDERED>(A.n, s, A.rp_re, A.col_re, A.val_re_df, A.rp_im, A.col_im, A.val_im_df, X, out, st);
 }
 }  // namespace
 
 void spmm_real_df(int64_t nrows, const int64_t* rp, const int32_t* col, const float2* val, const float4* X,
                   double2* Y, int s, cudaStream_t st) {
-  spmm_launch<SpDf<float4>>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X,
-                            OutRows<SpDf<float4>>{Y, nullptr, s}, st, true);
+  spmm_launch<SpDf<float4>, true>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X,
+                                  OutRows<SpDf<float4>>{Y, nullptr, s}, st);
 }
 
 void to_df(const double2* X, float4* Y, int64_t count, cudaStream_t st) {
@@ -93,19 +93,25 @@ void to_df(const double2* X, float4* Y, int64_t count, cudaStream_t st) {
 }
 
 void spmm_split_df(const DevSplitCsr& A, const float4* X, double2* Y, const double2* B, int s, cudaStream_t st) {
-  spmm_df(A, X, OutRows<SpDf<float4>>{Y, B, s}, s, st, B != nullptr);  // t = v - A q feeds FP32 local solves: in storage order
+  if (B)  // t = v - A q feeds FP32 local solves: in storage order
+    spmm_df<true>(A, X, OutRows<SpDf<float4>>{Y, B, s}, s, st);
+  else
+    spmm_df<false>(A, X, OutRows<SpDf<float4>>{Y, nullptr, s}, s, st);
 }
 void spmm_split_df_cols(const DevSplitCsr& A, const float4* X, double2* Y, int s, cudaStream_t st) {
-  spmm_df(A, X, OutCols<SpDf<float4>>{Y, A.n}, s, st);
+  spmm_df<false>(A, X, OutCols<SpDf<float4>>{Y, A.n}, s, st);
 }
 void spmm_split_df(const DevSplitCsr& A, const float4* X, float4* Y, int s, cudaStream_t st) {
-  spmm_df(A, X, OutDf<SpDf<float4>>{Y, s}, s, st);
+  spmm_df<false>(A, X, OutDf<SpDf<float4>>{Y, s}, s, st);
 }
 void spmm_split_df(const DevSplitCsr& A, const float2* X, double2* Y, int s, cudaStream_t st) {
-  spmm_df(A, X, OutRows<SpDf<float2>>{Y, nullptr, s}, s, st);
+  spmm_df<false>(A, X, OutRows<SpDf<float2>>{Y, nullptr, s}, s, st);
 }
 void spmm_split_df(const DevSplitCsr& A, const float2* X, float4* Y, int s, cudaStream_t st, bool ordered) {
-  spmm_df(A, X, OutDf<SpDf<float2>>{Y, s}, s, st, ordered);
+  if (ordered)
+    spmm_df<true>(A, X, OutDf<SpDf<float2>>{Y, s}, s, st);
+  else
+    spmm_df<false>(A, X, OutDf<SpDf<float2>>{Y, s}, s, st);
 }
 
 }  // namespace hz

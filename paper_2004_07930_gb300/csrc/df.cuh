@@ -98,15 +98,6 @@ static __device__ __forceinline__ void df_mac2(pair2& sh, pair2& sl, pair2 ah, p
   df_add2(sh, sl, np, fma2(al, xh, fma2(ah, xh, np)));
 }
 
-// (sh, sl) += (h, l)
-static __device__ __forceinline__ void df_add(float& sh, float& sl, float h, float l) {
-  const float t = __fadd_rn(sh, h);
-  const float z = __fsub_rn(t, sh);
-  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, z)), __fsub_rn(h, z));
-  sl = __fadd_rn(sl, __fadd_rn(err, l));
-  sh = t;
-}
-
 // renormalise (h, l) so that |l| is at most half an ulp of h (Fast2Sum; |h| >= |l| or h = 0)
 static __device__ __forceinline__ void df_norm(float& h, float& l) {
   const float t = __fadd_rn(h, l);

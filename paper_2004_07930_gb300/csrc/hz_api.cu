@@ -857,7 +857,6 @@ void ensure_workspace(hz_ctx* c, int s) {
   c->Xsub = (double2*)p.alloc<char>(c->lf.sub_rows * cols * ef);
   c->lf.mf.Wout = p.alloc<char>(c->lf.mf.rows_total * cols * ef);
   if (c->lf.mf.tc) c->lf.mf.P = p.alloc<char>((size_t)c->lf.mf.max_slots * MF_TILE_ROWS * cols * ef);
-  c->lf.mf.s_cap = s;
   // double-float Arnoldi for the outer space unless block FGMRES or recycling (which read W in FP64)
   alloc_krylov(c->Kout, n, s, c->opt.restart, p, c->st, false,
                c->df && !c->opt.block_arnoldi && c->opt.recycle == 0);
@@ -911,7 +910,6 @@ void ensure_workspace(hz_ctx* c, int s) {
     c->XsubH = (double2*)p.alloc<char>(c->lc.sub_rows * cols * ec);
     c->lc.mf.Wout = p.alloc<char>(c->lc.mf.rows_total * cols * ec);
     if (c->lc.mf.tc) c->lc.mf.P = p.alloc<char>((size_t)c->lc.mf.max_slots * MF_TILE_ROWS * cols * ec);
-    c->lc.mf.s_cap = s;
     if (c->opt.coarse_mode == HZ_COARSE_GMRES) {
       alloc_krylov(c->Kin, nh, s, std::max(1, c->opt.coarse_inner_its), p, c->st, c->coarse32, c->df);
       CK(cudaMemsetAsync(c->Kin.tol, 0, s * sizeof(double), c->st));

@@ -68,15 +68,18 @@ struct OutCols {  // Y = A X with the columns contiguous, [s][n]
 
 void spmm_split(const DevSplitCsr& A, const double2* X, double2* Y, const double2* B, int s, cudaStream_t st,
                 bool ordered) {
-  spmm_launch<SpF64>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im, A.val_im, X, OutRows{Y, B, s}, st, ordered);
+  if (ordered)
+    spmm_launch<SpF64, true>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im, A.val_im, X, OutRows{Y, B, s}, st);
+  else
+    spmm_launch<SpF64, false>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im, A.val_im, X, OutRows{Y, B, s}, st);
 }
 void spmm_split_cols(const DevSplitCsr& A, const double2* X, double2* Y, int s, cudaStream_t st) {
-  spmm_launch<SpF64>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im, A.val_im, X, OutCols{Y, A.n}, st);
+  spmm_launch<SpF64, false>(A.n, s, A.rp_re, A.col_re, A.val_re, A.rp_im, A.col_im, A.val_im, X, OutCols{Y, A.n}, st);
 }
 
 void spmm_real(int64_t nrows, const int64_t* rp, const int32_t* col, const double* val, const double2* X,
                double2* Y, int s, cudaStream_t st) {
-  spmm_launch<SpF64>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRows{Y, nullptr, s}, st, true);
+  spmm_launch<SpF64, true>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRows{Y, nullptr, s}, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -152,8 +152,7 @@ struct DevMF {
   void* M = nullptr;            // X_t factors (double2 or float2), grouped layout
   void* MT = nullptr;           // X_t^T (backward sweep), grouped layout
   void* Dinv = nullptr;         // 1/D (double2 or float2)
-  void* Wout = nullptr;         // front vectors [rows_total][s_cap]: y_P and parent updates
-  int s_cap = 0;
+  void* Wout = nullptr;         // front vectors [rows_total][sub_cols]: y_P and parent updates
   int* gidx = nullptr;          // [nsub_rows] global row of each sub-vector row (R_i)
   int* own = nullptr;           // [n] sub-vector row of the owning copy (D_i Boolean)
   int* perturbed = nullptr;     // device counter
@@ -170,7 +169,7 @@ struct DevMF {
   int4* frb = nullptr;             // (front, first row, tiles, first slot)
   int4* brb = nullptr;
   int64_t max_slots = 0;           // partial-result slots of the largest level
-  void* P = nullptr;               // partial tile results [max_slots][128][s_cap]
+  void* P = nullptr;               // partial tile results [max_slots][128][sub_cols]
   int* fs_ptr_h = nullptr;      // host [nlevels+1] forward SIMT tiles per level (tensor-core mode)
   int* bs_ptr_h = nullptr;      // host [nlevels+1] backward SIMT tiles per level
   int* ftc_ptr_h = nullptr;     // host [nlevels+1] forward tensor-core tiles per level

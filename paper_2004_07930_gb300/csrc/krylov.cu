@@ -589,11 +589,11 @@ struct OutRowsF {  // Y = A X, or B - A X
 }  // namespace
 
 void spmm_split_f32(const DevSplitCsr& A, const float2* X, float2* Y, int s, cudaStream_t st, const float2* B) {
-  spmm_launch<SpF32>(A.n, s, A.rp_re, A.col_re, A.val_re_f, A.rp_im, A.col_im, A.val_im_f, X, OutRowsF{Y, B, s}, st, true);
+  spmm_launch<SpF32, true>(A.n, s, A.rp_re, A.col_re, A.val_re_f, A.rp_im, A.col_im, A.val_im_f, X, OutRowsF{Y, B, s}, st);
 }
 void spmm_real_f32(int64_t nrows, const int64_t* rp, const int32_t* col, const float* val, const float2* X,
                    float2* Y, int s, cudaStream_t st) {
-  spmm_launch<SpF32>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRowsF{Y, nullptr, s}, st, true);
+  spmm_launch<SpF32, true>(nrows, s, rp, col, val, nullptr, nullptr, nullptr, X, OutRowsF{Y, nullptr, s}, st);
 }
 
 __global__ void k_d2f(const double2* __restrict__ X, float2* __restrict__ Y, int64_t count) {

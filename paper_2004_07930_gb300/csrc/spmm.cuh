@@ -43,7 +43,7 @@ struct SpF64 {
   }
   static __device__ __forceinline__ double2 to_d(Acc a) { return a; }
 };
-struct SpF32 {
+struct SpF32 {  // ordered sums only
   using Val = float;
   using X = float2;
   using Acc = float2;
@@ -55,10 +55,6 @@ struct SpF32 {
   static __device__ __forceinline__ void im(Acc& y, Val b, X x) {
     y.x = fmaf(-b, x.y, y.x);
     y.y = fmaf(b, x.x, y.y);
-  }
-  static __device__ __forceinline__ Acc add(Acc a, Acc b) { return make_float2(a.x + b.x, a.y + b.y); }
-  static __device__ __forceinline__ Acc shfl(Acc a, int off) {
-    return make_float2(__shfl_down_sync(0xffffffffu, a.x, off), __shfl_down_sync(0xffffffffu, a.y, off));
   }
 };
 // Double-float values, the real and the imaginary part side by side in packed
@@ -201,11 +197,12 @@ __global__ void __launch_bounds__(256, CPT == 1 ? 5 : 4) k_spmm(int64_t n, int s
     sp_row<P, false, T>(y, rp_re[r] + t, rp_re[r + 1], col_re, val_re, X + c, dc, pitch);
     if (rp_im) sp_row<P, true, T>(y, rp_im[r] + t, rp_im[r + 1], col_im, val_im, X + c, dc, pitch);
   }
+  if constexpr (T > 1)
 #pragma unroll
-  for (int o = T / 2; o > 0; o /= 2) {
-    const typename P::Acc z = P::shfl(y[0], o * s);
-    if (t < o) y[0] = P::add(y[0], z);
-  }
+    for (int o = T / 2; o > 0; o /= 2) {
+      const typename P::Acc z = P::shfl(y[0], o * s);
+      if (t < o) y[0] = P::add(y[0], z);
+    }
   if (r < n && t == 0) out(r, c, y[0]);
   if (CPT == 2 && dc > 0) out(r, c + dc, y[CPT - 1]);
 }
@@ -257,34 +254,33 @@ void spmm_launch_t(int64_t n, int s, const int64_t* rp_re, const int32_t* col_re
 // Lanes per row: as many as fit a warp, up to 8, while the block has fewer
 // entries than the SMs have lanes to give them (cube of 6^3 cells, one column,
 // FP64: 15 us with one lane, 6 with eight); on large blocks two to four where
-// a row's s columns leave the index and value loads uncoalesced. `ordered`:
+// a row's s columns leave the index and value loads uncoalesced. ORDERED:
 // one lane per row, every row summed in storage order (the operators of the
 // inner coarse iteration, whose rounding the preconditioner amplifies).
-template <typename P, typename Out>
+template <typename P, bool ORDERED, typename Out>
 void spmm_launch(int64_t n, int s, const int64_t* rp_re, const int32_t* col_re, const typename P::Val* val_re,
                  const int64_t* rp_im, const int32_t* col_im, const typename P::Val* val_im, const typename P::X* X,
-                 Out out, cudaStream_t st, bool ordered = false) {
+                 Out out, cudaStream_t st) {
   if (n * s == 0) return;
   const bool small = n * s < 160000;
-  if constexpr (std::is_same<P, SpF64>::value)
-    if (ordered && small) {
+  if constexpr (ORDERED && std::is_same<P, SpF64>::value)
+    if (small) {
       k_spmm_parts<<<(unsigned)((2 * n * s + 63) / 64), 64, 0, st>>>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im,
                                                                    reinterpret_cast<const double*>(X), out);
       count_launch();
       return;
     }
-  const int fit = s <= 4 ? 8 : (s <= 8 ? 4 : (s <= 16 ? 2 : 1));
-  const int T = ordered ? 1 : (small ? fit : (s <= 2 ? 4 : (s <= 4 ? 2 : 1)));
-  if (T == 8)
-    spmm_launch_t<P, 8, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
-  else if (T == 4)
-    spmm_launch_t<P, 4, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
-  else if (T == 2)
-    spmm_launch_t<P, 2, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
-  else if (!std::is_same<P, SpF64>::value && s >= SP_COL && n * s >= SP_LARGE)
-    spmm_launch_t<P, 1, 2>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
-  else
-    spmm_launch_t<P, 1, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
+  if constexpr (!ORDERED) {
+    const int fit = s <= 4 ? 8 : (s <= 8 ? 4 : (s <= 16 ? 2 : 1));
+    const int T = small ? fit : (s <= 2 ? 4 : (s <= 4 ? 2 : 1));
+    if (T == 8) return spmm_launch_t<P, 8, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
+    if (T == 4) return spmm_launch_t<P, 4, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
+    if (T == 2) return spmm_launch_t<P, 2, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
+  }
+  if constexpr (!std::is_same<P, SpF64>::value)
+    if (s >= SP_COL && n * s >= SP_LARGE)
+      return spmm_launch_t<P, 1, 2>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
+  spmm_launch_t<P, 1, 1>(n, s, rp_re, col_re, val_re, rp_im, col_im, val_im, X, out, st);
 }
 
 }  // namespace hz
