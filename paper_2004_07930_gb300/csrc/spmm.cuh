@@ -8,8 +8,9 @@
 // their parts at the end.
 //
 // What bounds it, on the 5 Hz workload (0.95M rows, 43.7M nonzeros, 16 columns,
-// double-float, 1.06 ms with both transposes; one thread per column and row,
-// rows in their order, scalar arithmetic: 1.28): the FMA pipe's two cycles per
+// double-float, 1.06 ms with the input's transpose, the output's columns
+// written here; one thread per column and row, rows in their order, scalar
+// arithmetic: 1.28): the FMA pipe's two cycles per
 // packed instruction (0.45 ms) next to the latency of the X rows, half of
 // which come from L2. DRAM has 0.8 GB to move, 0.12 ms.
 #pragma once
@@ -138,7 +139,8 @@ constexpr int SP_COL = 16;
 constexpr int64_t SP_LARGE = 400000;
 
 // The CTA's rows in the order of their length, by runs of 32: threadIdx.y's
-// row. Rows of a quadratic space have 20 to 65 nonzeros, and a warp of two to
+// row. Rows of the cubic space have 20 (a node of one boundary face) to 175
+// nonzeros (a vertex), 45 on average, and a warp of two to
 // ten rows works as long as its longest (25 of 32 lanes busy on average in
 // their own order with two, 20 with four).
 __device__ __forceinline__ int sp_rank(int64_t n, int s, const int64_t* __restrict__ rp) {
