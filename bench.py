@@ -38,13 +38,13 @@ sys.path.insert(0, ROOT)
 
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FP64_NOMINAL_GFLOPS = 1250.0  # nominal GB300 FP64 rate, context only (the FP64 peak is measured live)
-TILE_PROFILE = os.path.join(ROOT, "profiles", "k_mf_tile_overthrust5_quarter.md")
+TILE_PROFILE = os.path.join(ROOT, "profiles", "k_sweep_level_overthrust5_quarter.md")
 
 
 def fronts_traffic(cfg, per_app):
     """DRAM bytes of one application of the fine local solves: the ratio of
     DRAM traffic to algorithmic bytes that ncu measured on the quarter crop
-    (profiles/k_mf_tile_overthrust5_quarter.md) times this run's algorithmic
+    (profiles/k_sweep_level_overthrust5_quarter.md) times this run's algorithmic
     bytes; None when the profile is absent or for the cube, whose factors
     fit in L2."""
     if cfg == "cube":
@@ -730,7 +730,7 @@ def main():
         # a sweep reads each factor entry once per application: HBM is the roof of the
         # tensor-core form; the SIMT FP32 rate (16 flops per factor byte at s = 16) is given beside it
         roof = {"bound": "hbm", "achieved": hbm_achieved, "peak": hbm, "unit": "GB/s", "frac": hbm_achieved / hbm,
-                "traffic": None if tc_on else fronts_traffic(args.config, per_app),
+                "traffic": None if tc_on or pers else fronts_traffic(args.config, per_app),
                 "traffic_unit": "DRAM bytes per application of the fine local solves",
                 "kernel": kern, "peak_kind": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)",
                 "algorithmic_bytes_per_application": per_app, "applications": ph["calls"],

@@ -33,7 +33,9 @@
 // columns) the FP32 FMA pipe: 444M factor entries, 114 GFLOP per
 // application, 1.5 ms at the pipe's 74.8 TFLOP/s; with one column HBM: 7.1 GB,
 // 1.05 ms. Measured, whole preconditioner: 4.05 ms (tiles of 128 rows,
-// one or a quarter of one per thread: 7.16) and 1.69 ms (2.00). The leaf level runs at
+// one or a quarter of one per thread: 7.16) and 1.66 ms (2.00). With one column
+// eight of a warp's lanes hold distinct rows and each row's sum is one chain
+// in order, so that short levels wait for that chain (see k_sweep_long). The leaf level runs at
 // 52-55 % of the pipe; the middle levels, 1-10 K small fronts each, spend
 // 30-55 us on the latency of task, indices, inputs and factors in turn.
 //
@@ -663,7 +665,7 @@ __global__ void __launch_bounds__(SW_THREADS, sw_min_blocks<V, S, FWD, STREAM>()
 // ---------------------------------------------------------------------------
 constexpr int LG_KC = 32;                       // indices per ring stage (4 KB)
 constexpr int LG_NST = 2;                       // ring stages per warp
-constexpr unsigned LG_TASKS = 608;
+constexpr unsigned LG_TASKS = 608;              // levels of fewer tasks
 constexpr int LG_STAGE = LG_KC * MF_GR;         // entries per stage
 constexpr int LG_ROWS = SW_NW * MF_CHUNK;       // input rows of a window, one chunk per warp
 constexpr int LG_RPT = LG_ROWS / SW_THREADS;    // rows per thread
