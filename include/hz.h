@@ -113,8 +113,9 @@ typedef struct hz_options {
                                needs max_block <= 32. Servers keep one Krylov space per column */
   int32_t persistent_sweeps;/* 1: each SIMT front sweep is one launch over all tree levels (resident CTAs take
                                tasks in level order and wait for the fronts they depend on); 0 (default): one
-                               launch per level, with the same results to the bit; on large trees and in the
-                               mixed form the faster of the two. The tensor-core tiles keep one launch per level */
+                               launch per level, with the same results to the bit. Which is faster depends on
+                               the block and the tree; one column in the mixed form on all but small trees, and
+                               the tensor-core tiles, keep one launch per level */
   int32_t factor_fp32;      /* mixed form only. 1 (default): the fine fronts are factorised (partial LDL^T and
                                partitioned inverse) in complex FP32; 0: in FP64, then rounded to FP32. The
                                coarse fronts are factorised in FP64 in both forms */

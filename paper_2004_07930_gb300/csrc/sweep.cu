@@ -1003,7 +1003,12 @@ void solve_v(DevMF& mf, V* Xsub, int cols, cudaStream_t st) {
   A.Xsub = Xsub;
   A.Wout = (V*)mf.Wout;
   A.s = cols;
-  if (mf.persistent) {
+  // One FP32 column on a tree that fills the SMs goes level by level in either
+  // case: the persistent form keeps the chains that k_sweep_long cuts (cube of
+  // 6^3 cells 0.141 ms to 0.110, quarter workload 0.84 to 0.61, 5 Hz 2.65 to
+  // 1.74). Trees of fewer tasks gain from the launches saved (two-level, cube,
+  // with its coarse level of 1000 dofs level by level 1.87 ms, persistent 1.80).
+  if (mf.persistent && !(sizeof(V) == 8 && cols == 1 && mf.ftask_ptr_h[mf.nlevels] >= (int)LG_TASKS)) {
     auto both = [&](auto w) {
       sweep_all<V, decltype(w)::value, true>(mf, A, st);
       sweep_all<V, decltype(w)::value, false>(mf, A, st);
